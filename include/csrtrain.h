@@ -68,7 +68,8 @@ extern "C" {
 #define CSRT_DEV_INVALID 8    /* csrt_validate_csr found a broken invariant */
 
 /* weight_grad_dense precision. */
-#define CSRT_PREC_FP32 0      /* float32 FMA on the CUDA cores */
+#define CSRT_PREC_FP32 0      /* float32 accuracy: FMA on the CUDA cores, or float32 factors split into
+                                 three bf16 parts on tcgen05 (error below the FMA chain's) */
 #define CSRT_PREC_TF32 1      /* tcgen05 tensor cores, kind::tf32, float32 accumulate */
 
 /*
@@ -242,7 +243,10 @@ int spmm_fwd_noalloc_status(int32_t *flags, int32_t clear, void *stream);
  * matrix w - eta*G of Section 3.3 needs G at all M x K entries).
  * G[i, j] = sum_c dY[i, c] X[j, c]; dY is m x n, X is k x n, G is m x k,
  * all row-major. No 1/n factor is applied. precision: CSRT_PREC_FP32 or
- * CSRT_PREC_TF32 (operands rounded to TF32, float32 accumulation). */
+ * CSRT_PREC_TF32 (operands rounded to TF32, float32 accumulation).
+ * CSRT_PREC_FP32 uses the workspace, where it is large enough, for the bf16
+ * parts of dY and X; without one every shape runs on the CUDA cores (long
+ * reductions over few outputs need it, as before). */
 int weight_grad_dense(const float *dy, const float *x, int32_t m, int32_t k, int32_t n,
                       float *g, int32_t precision, void *ws, size_t ws_bytes, void *stream);
 

@@ -109,6 +109,8 @@ __global__ void split_reduce_kernel(const float *__restrict__ part, int64_t coun
 
 int gemm_tc_tf32(const float *dy, const float *x, int32_t m, int32_t k, int32_t n, float *g, void *ws,
                  size_t ws_bytes, cudaStream_t s, bool *handled);
+int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_t n, float *g, void *ws,
+                   size_t ws_bytes, cudaStream_t s, bool *handled);
 
 }  // namespace csrt
 
@@ -132,6 +134,11 @@ extern "C" int weight_grad_dense(const float *dy, const float *x, int32_t m, int
         int rc = gemm_tc_tf32(dy, x, m, k, n, g, ws, ws_bytes, s, &handled);
         if (rc || handled) return rc;
         // shapes the tensor-core kernel does not take fall through to FP32
+    }
+    if (precision == CSRT_PREC_FP32) {
+        bool handled = false;
+        int rc = gemm_split_f32(dy, x, m, k, n, g, ws, ws_bytes, s, &handled);
+        if (rc || handled) return rc;
     }
     const GemmSplit sp = gemm_split(m, k, n);
     float *out = g;

@@ -1,0 +1,422 @@
+// Dense weight gradient G = dY X^T in float32 accuracy on the tensor cores.
+//
+// Every float32 factor is the sum of three bf16 parts, x = x1 + x2 + x3 with
+// 8 significant bits each (round to nearest of what is left, so |x2| <= 2^-9
+// |x|, |x3| <= 2^-18 |x| and the sum is exact up to 2^-26 |x|). The product
+// is taken as x1 y1 + x1 y2 + x2 y1 + x2 y2 + x1 y3 + x3 y1; what is left out
+// is below 2^-26 |x y|, under float32's own rounding unit 2^-24.
+//
+// The accumulation must not lose what the split keeps. tcgen05.mma adds into
+// its float32 accumulator with truncation (measured: 2 bits beyond the
+// accumulator's last place are kept, the sum is cut toward zero), so a long
+// chain drifts: over 256 columns 2.3e-7 of the result against 1.1e-7 for a
+// chain of fused multiply-adds. Hence the reduction runs in chunks of 32
+// columns: in each the five small products come first (their truncations are
+// 2^-8 smaller), then the two steps of x1 y1, and the chunk's sum is added to
+// a float32 register accumulator with round to nearest. The error against 64
+// bits is then below the fused multiply-add chain's for every n.
+//
+//  split_rows_kernel       dY and X to their planes (bf16, [3][rows][ld]) in the
+//                          workspace, a warp per row; rows that hold a value of
+//                          2^60 or more, an infinity or a NaN are marked.
+//  gemm_split_kernel       CTA pairs (cta_group::2) walk 256 x 256 tiles of G:
+//                          per 64 columns six 16 KB slices per CTA (three planes
+//                          of its 128 rows of dY and 128 rows of X) by TMA, per
+//                          chunk 12 MMAs of M = 256, N = 256, K = 16; two accumulators
+//                          in tensor memory alternate between chunks; sixteen
+//                          warps per CTA read them back and keep the sums of
+//                          their 32 rows x 64 columns in registers.
+// Entries of marked rows are computed again by the epilogue with the plain
+// float32 chain, so infinities and NaN give what they give there.
+//
+// What bounds it: six bf16 products per multiply-add; 4096 x 4096 x 256 is
+// 51.5 GFLOP of MMA, 27 us at the measured bf16 rate, and 3.4 waves of tiles
+// run as 4. Measured (GB300, inputs in L2): 4096 x 4096 x 250 57.6 us (the
+// CUDA-core kernel 381), 4096 x 9216 x 256 107 us (830), 4096 x 4096 x 1024
+// 179 us (1464), 1000 x 4096 x 256 19 us (110). The MMAs alone take 0.91 us
+// per chunk and wave, with the operand loads and the reading back 1.15; a
+// wave's stores, which the next tile's first two chunks hide in part, 2-3 us.
+// 64-byte operand rows (stages of 32 columns) ran 11% slower than 128-byte
+// ones, eight reading warps with 128 sums each (spilling) 10%.
+#include "tc_pair.cuh"
+
+namespace csrt {
+
+constexpr int kGsChunk = 32;                           // reduction columns per chunk sum
+constexpr int kGsStageCols = 64;                       // per pipeline stage: rows of 128 bytes
+constexpr int kGsSlice = 128 * kGsStageCols * 2;       // one plane of 128 rows: 16 KB
+constexpr int kGsStageBytes = 6 * kGsSlice;            // three planes of each operand
+constexpr int kGsStages = 2;
+constexpr int kGsEpiWarps = 16;                        // per TMEM lane quarter four, 64 columns each
+constexpr int kGsEpiCols = 64;
+constexpr int kGsProd = 4;                             // a warpgroup of producers (TMA, MMA, two idle)
+constexpr int kGsThreads = 32 * (kGsProd + kGsEpiWarps);
+// register split within the launch's 640 x 96: the sums (64), a block read
+// back (32) and addresses need more than 96 in the epilogue warps
+constexpr int kGsProdRegs = 32, kGsEpiRegs = 112;
+static_assert(128 * kGsProdRegs + 32 * kGsEpiWarps * kGsEpiRegs <= kGsThreads * 96, "register split");
+constexpr int kGsTile = 256;
+constexpr int kGsStageOut = 32 * 16 * 4;               // a 32 x 16 block on its way out
+constexpr int kGsSmem = kGsStages * kGsStageBytes + kGsEpiWarps * kGsStageOut + 1024 + 256;
+static_assert(kGsSmem <= 232448, "shared memory per block");
+constexpr uint32_t kGsIdesc = idesc_f16(1, 256, 256);
+
+struct GsArgs {
+    float *g;
+    int32_t m, k, n;
+    const float *dy, *x;             // the float32 operands (marked rows)
+    const uint8_t *bad_dy, *bad_x;   // marked rows
+    int32_t tiles_k, num_tiles;
+    WsHeader *hdr;
+};
+
+// Planes of rows 0..m-1 of dY and 0..k-1 of X (one warp per row, eight
+// columns per lane and step).
+__global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict__ dy, const float *__restrict__ x,
+                                                         int32_t m, int32_t k, int32_t n, int32_t ld,
+                                                         __nv_bfloat16 *__restrict__ pdy,
+                                                         __nv_bfloat16 *__restrict__ px, uint8_t *__restrict__ bad_dy,
+                                                         uint8_t *__restrict__ bad_x, int vec) {
+    pdl_enter();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the GEMM's set-up may begin
+    const int lane = threadIdx.x & 31;
+    int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (r >= (int64_t)m + k) return;
+    const bool is_x = r >= m;
+    if (is_x) r -= m;
+    const int64_t rows = is_x ? k : m;
+    const float *src = (is_x ? x : dy) + r * n;
+    __nv_bfloat16 *dst = (is_x ? px : pdy) + r * ld;
+    const int64_t plane = rows * ld;
+    bool bad = false;
+    for (int c = lane * 8; c < n; c += 256) {
+        float v[8];
+        if (vec && c + 8 <= n) {
+            const float4 a = ldg_f4(src + c), b = ldg_f4(src + c + 4);
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = c + e < n ? __ldg(src + c + e) : 0.f;
+        }
+        __nv_bfloat162 p[3][4];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            const float2 a = make_float2(v[e], v[e + 1]);
+            if (!(fabsf(a.x) < 0x1p60f) || !(fabsf(a.y) < 0x1p60f)) bad = true;
+            const __nv_bfloat162 b1 = __float22bfloat162_rn(a);
+            const float2 f1 = __bfloat1622float2(b1);
+            const float2 r1 = make_float2(a.x - f1.x, a.y - f1.y);
+            const __nv_bfloat162 b2 = __float22bfloat162_rn(r1);
+            const float2 f2 = __bfloat1622float2(b2);
+            p[0][e / 2] = b1;
+            p[1][e / 2] = b2;
+            p[2][e / 2] = __float22bfloat162_rn(make_float2(r1.x - f2.x, r1.y - f2.y));
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4 *>(dst + q * plane + c) = *reinterpret_cast<uint4 *>(p[q]);
+    }
+    const bool any = __any_sync(0xffffffffu, bad);
+    if (lane == 0) (is_x ? bad_x : bad_dy)[r] = any ? 1 : 0;
+}
+
+__global__ void __launch_bounds__(kGsThreads, 1)
+    gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, GsArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    float *epi = reinterpret_cast<float *>(smem + kGsStages * kGsStageBytes);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kGsStages * kGsStageBytes + kGsEpiWarps * kGsStageOut);
+    uint64_t *empty = full + kGsStages;
+    uint64_t *accf = empty + kGsStages;   // [2] chunk sums ready
+    uint64_t *acce = accf + 2;            // [2] read back (the leader's: all warps of both CTAs)
+    uint64_t *fin = acce + 2;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
+    __shared__ volatile int s_abort;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    const int num_kb = (a.n + kGsStageCols - 1) / kGsStageCols;
+    const int num_ch = (a.n + kGsChunk - 1) / kGsChunk;
+
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        for (int s = 0; s < kGsStages; ++s) {
+            mbar_init(full + s, 1);
+            mbar_init(empty + s, 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(accf + b, 1);
+            mbar_init(acce + b, 2 * kGsEpiWarps);
+        }
+        mbar_init(fin, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync_all();   // the barriers of both CTAs are set up
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+    // nothing before this reads or writes global memory: the set-up overlaps
+    // the end of the split kernel, whose planes are complete from here on
+    pdl_enter();
+
+    if (warp < kGsProd) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGsProdRegs));
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            for (int t = pair; t < a.num_tiles && !s_abort; t += pairs) {
+                const int m0 = (t / a.tiles_k) * kGsTile + (int)rank * 128;
+                const int k0 = (t % a.tiles_k) * kGsTile + (int)rank * 128;
+                for (int kb = 0; kb < num_kb; ++kb, ++it) {
+                    const int s = it % kGsStages;
+                    if (!mbar_wait_or_abort(empty + s, ((it / kGsStages) & 1) ^ 1, &s_abort)) break;
+                    if (rank == 0) mbar_expect_tx(full + s, 2 * kGsStageBytes);
+                    const uint32_t bar = map_to_rank(full + s, 0);
+                    uint8_t *st = smem + s * kGsStageBytes;
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        tma_load_2d_pair(st + p * kGsSlice, &map_a, kb * kGsStageCols, p * a.m + m0, bar);
+                        tma_load_2d_pair(st + (3 + p) * kGsSlice, &map_b, kb * kGsStageCols, p * a.k + k0, bar);
+                    }
+                }
+            }
+            // every load of both CTAs must land before the pair may exit
+            if (rank == 0)
+                for (int i = imax(0, it - kGsStages); i < it; ++i)
+                    mbar_wait(full + i % kGsStages, (i / kGsStages) & 1);
+        }
+    } else if (warp == 1) {
+        if (rank == 0 && lane == 0) {
+            int it = 0, ch = 0;
+            for (int t = pair; t < a.num_tiles && !s_abort; t += pairs) {
+                for (int kb = 0; kb < num_kb; ++kb, ++it) {
+                    const int s = it % kGsStages;
+                    const uint8_t *st = smem + s * kGsStageBytes;
+                    if (!mbar_wait_or_abort(full + s, (it / kGsStages) & 1, &s_abort)) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const int halves = imin(2, num_ch - 2 * kb);
+                    for (int hf = 0; hf < halves; ++hf, ++ch) {
+                        const int b = ch & 1;
+                        if (!mbar_wait_pair(acce + b, ((ch >> 1) & 1) ^ 1, &s_abort)) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t d = tmem + (uint32_t)(b * 256);
+                        // planes of (dY, X): the small products first
+                        const int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+                        for (int q = 0; q < 6; ++q)
+#pragma unroll
+                            for (int k = 0; k < kGsChunk / 16; ++k)
+                                mma_f16_pair(d, smem_desc_sw128(st + pa[q] * kGsSlice + hf * 64 + k * 32),
+                                             smem_desc_sw128(st + (3 + pb[q]) * kGsSlice + hf * 64 + k * 32), kGsIdesc,
+                                             (q > 0 || k > 0) ? 1u : 0u);
+                        if (hf == halves - 1) mma_commit_pair(empty + s);
+                        mma_commit_pair(accf + b);
+                    }
+                }
+            }
+            asm volatile(
+                "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(fin))
+                : "memory");
+            mbar_wait(fin, 0);   // nothing of ours still runs on the tensor cores
+        }
+    }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kGsEpiRegs));
+        const int q = warp & 3;                  // TMEM lanes 32q ..: rows 32q .. of this CTA's 128
+        const int h = (warp - kGsProd) >> 2;     // column quarter of the tile
+        const uint32_t acce0 = map_to_rank(acce, 0), acce1 = map_to_rank(acce + 1, 0);
+        float *xb = epi + (warp - kGsProd) * (kGsStageOut / 4);
+        int it = 0;
+        for (int t = pair; t < a.num_tiles; t += pairs) {
+            const int64_t row = (int64_t)(t / a.tiles_k) * kGsTile + rank * 128 + q * 32 + lane;
+            const int64_t col0 = (int64_t)(t % a.tiles_k) * kGsTile + h * kGsEpiCols;
+            float acc[kGsEpiCols];
+            bool ok = true;
+            for (int kb = 0; kb < num_ch; ++kb, ++it) {
+                const int b = it & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait_or_abort(accf + b, (it >> 1) & 1, &s_abort));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int c = 0; c < kGsEpiCols; c += 32) {
+                    uint32_t r[32];
+                    tmem_ld_32cols(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256 + h * kGsEpiCols + c), r);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        acc[c + e] = kb == 0 ? __uint_as_float(r[e]) : acc[c + e] + __uint_as_float(r[e]);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(b ? acce1 : acce0);
+            }
+            if (!ok) break;
+            if (a.k % 8 == 0 && (reinterpret_cast<uintptr_t>(a.g) & 31) == 0) {
+                // lane = row holds 64 columns; groups of four lanes exchange
+                // 32-byte units so that lane j of a group holds unit j of each
+                // of the group's rows: a store then covers eight whole lines
+                // instead of a sector of 32 (4096 x 4096 x 32 27 -> 25 us)
+                const int j = lane & 3;
+#pragma unroll
+                for (int c = 0; c < kGsEpiCols; c += 32) {
+#pragma unroll
+                    for (int sft = 1; sft <= 2; sft <<= 1) {
+                        const bool up = (j & sft) != 0;
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+                            if (p & sft) continue;
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                float &lo = acc[c + p * 8 + e], &hi = acc[c + (p | sft) * 8 + e];
+                                const float got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, sft);
+                                if (up) lo = got;
+                                else hi = got;
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const int64_t r = row - j + p, col = col0 + c + j * 8;
+                        if (r < a.m && col < a.k) st_global_f8(a.g + r * a.k + col, acc + c + p * 8);
+                    }
+                }
+            } else {
+                // any alignment: 32 x 16 blocks through shared memory, two
+                // rows per store (16-byte chunk i of row r at i ^ ((r >> 1) & 3))
+#pragma unroll
+                for (int c = 0; c < kGsEpiCols; c += 16) {
+                    __syncwarp();
+#pragma unroll
+                    for (int e = 0; e < 16; e += 4)
+                        *reinterpret_cast<float4 *>(xb + lane * 16 + (e ^ (((lane >> 1) & 3) << 2))) =
+                            make_float4(acc[c + e], acc[c + e + 1], acc[c + e + 2], acc[c + e + 3]);
+                    __syncwarp();
+                    const int cc = lane & 15;
+                    const int64_t col = col0 + c + cc;
+                    const int64_t rb = row - lane + (lane >> 4);
+#pragma unroll 4
+                    for (int i = 0; i < 32; i += 2) {
+                        const int r = i + (lane >> 4);
+                        if (rb + i < a.m && col < a.k) a.g[(rb + i) * a.k + col] = xb[r * 16 + (cc ^ (((r >> 1) & 3) << 2))];
+                    }
+                }
+            }
+            // entries of marked rows: the float32 chain
+            const bool bad_row = row < a.m && a.bad_dy[row];
+            bool bad_col = false;
+#pragma unroll
+            for (int e = 0; e < kGsEpiCols / 32; ++e) {
+                const int64_t col = col0 + e * 32 + lane;
+                bad_col |= col < a.k && a.bad_x[col];
+            }
+            if (__any_sync(0xffffffffu, bad_row || bad_col)) {
+                __syncwarp();
+                const int cols = (int)imin<int64_t>(kGsEpiCols, a.k - col0);
+                for (int e = 0; e < cols; ++e)
+                    if (row < a.m && (bad_row || a.bad_x[col0 + e])) {
+                        const float *p = a.dy + row * a.n, *w = a.x + (col0 + e) * a.n;
+                        float s = 0.f;
+                        for (int c = 0; c < a.n; ++c) s = fmaf(__ldg(p + c), __ldg(w + c), s);
+                        a.g[row * a.k + col0 + e] = s;
+                    }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && s_abort) {
+        dev_flag(a.hdr, CSRT_DEV_TIMEOUT);
+        a.hdr->timeout_site = 11;
+    }
+    cluster_sync_all();   // no CTA leaves while the other may still use its shared memory
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
+static int64_t gs_ld(int32_t n) { return ceil_div<int64_t>(n, 8) * 8; }
+static size_t gs_align(size_t v) { return (v + 255) / 256 * 256; }
+
+// Scratch of an m x k gradient over n columns: the planes and the marks.
+static size_t gs_bytes(int64_t m, int64_t k, int32_t n) {
+    return gs_align((size_t)(6 * m * gs_ld(n))) + gs_align((size_t)(6 * k * gs_ld(n))) + gs_align((size_t)m) +
+           gs_align((size_t)k) + 256;
+}
+
+size_t gemm_split_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
+    if (rows < 64 || cols < 64) return 0;
+    const size_t cap = max_n <= 16384 ? (size_t)256 << 20 : (size_t)64 << 20;
+    return imin(gs_bytes(rows, cols, max_n), cap);
+}
+
+int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_t n, float *g, void *ws,
+                   size_t ws_bytes, cudaStream_t s, bool *handled) {
+    *handled = false;
+    // under 32 columns a chain of multiply-adds is as exact (16 columns: 4.3e-8
+    // against 4.7e-8) and its time is launch latency either way
+    if (m < 64 || k < 64 || n < kGsChunk || !device_is_sm10x()) return CSRT_OK;
+    if (ws == nullptr || ws_bytes < kWsReservedBytes + gs_bytes(m, k, n)) return CSRT_OK;
+    const int tiles_k = (int)ceil_div<int64_t>(k, kGsTile);
+    const int tiles = (int)ceil_div<int64_t>(m, kGsTile) * tiles_k;
+    const int pairs = imin(tiles, imax(1, num_sms() / 2));
+    // Where the CUDA-core kernel is still faster: small outputs, few columns.
+    // Both times fitted to measurements on GB300 (microseconds; the split
+    // GEMM within 15% over 64..4096 x 64..9216 x 32..1024, the CUDA-core
+    // kernel, a latency per column or its 22 TFLOP/s, likewise).
+    const double waves = (double)ceil_div(tiles, pairs), chunks = (double)ceil_div(n, kGsChunk);
+    const double t_split = 9.5 + waves * (2.8 + 1.15 * chunks);
+    const double t_fma = imax(2.6 + 0.1 * imin(n, 512), 2.0 * m * k * n / 22e6);
+    if (t_split > t_fma) return CSRT_OK;
+    const int32_t ld = (int32_t)gs_ld(n);
+    char *p = ws_scratch(ws);
+    p = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(p) + 255) & ~uintptr_t(255));
+    __nv_bfloat16 *pdy = reinterpret_cast<__nv_bfloat16 *>(p);
+    p += gs_align((size_t)6 * m * ld);
+    __nv_bfloat16 *px = reinterpret_cast<__nv_bfloat16 *>(p);
+    p += gs_align((size_t)6 * k * ld);
+    uint8_t *bad_dy = reinterpret_cast<uint8_t *>(p);
+    uint8_t *bad_x = bad_dy + gs_align((size_t)m);
+    CUtensorMap ma, mb;
+    if (!make_map16(&ma, pdy, true, (int64_t)3 * m, n, ld, 128, kGsStageCols) ||
+        !make_map16(&mb, px, true, (int64_t)3 * k, n, ld, 128, kGsStageCols))
+        return CSRT_OK;
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    CSRT_CHECK_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return CSRT_OK;
+    if (!attr_set[dev]) {
+        CSRT_CHECK_CUDA(cudaFuncSetAttribute(gemm_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGsSmem));
+        attr_set[dev] = true;
+    }
+    GsArgs a;
+    a.g = g;
+    a.m = m;
+    a.k = k;
+    a.n = n;
+    a.dy = dy;
+    a.x = x;
+    a.bad_dy = bad_dy;
+    a.bad_x = bad_x;
+    a.tiles_k = tiles_k;
+    a.num_tiles = tiles;
+    a.hdr = static_cast<WsHeader *>(ws);
+    const int vec = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(dy) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
+    launch_pdl(split_rows_kernel, dim3((unsigned)ceil_div<int64_t>((int64_t)m + k, 8)), dim3(256), 0, s, dy, x, m, k, n,
+               ld, pdy, px, bad_dy, bad_x, vec);
+    launch_pair(gemm_split_kernel, (unsigned)(2 * pairs), kGsThreads, kGsSmem, s, ma, mb, a);
+    count_launch(2);
+    *handled = true;
+    return check_launch("gemm_split_kernel");
+}
+
+}  // namespace csrt

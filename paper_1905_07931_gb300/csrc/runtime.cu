@@ -59,6 +59,8 @@ int csrt_workspace_bytes(int32_t rows, int32_t cols, int32_t max_n, size_t *byte
     if (t > need) need = t;
     t = gemm_scratch_bytes(rows, cols, max_n);
     if (t > need) need = t;
+    t = gemm_split_scratch_bytes(rows, cols, max_n);
+    if (t > need) need = t;
     t = fused_prox_scratch_bytes(rows, cols);
     if (t > need) need = t;
     *bytes = kWsReservedBytes + ((need + 255) / 256) * 256;

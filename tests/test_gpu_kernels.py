@@ -320,6 +320,40 @@ def test_weight_grad_dense(C, m, k, n, prec):
                  what=f"weight_grad_dense prec={prec}")
 
 
+@pytest.mark.parametrize("m,k,n", [(300, 520, 250),      # ragged rows, tiles and columns
+                                   (257, 1027, 200),     # one row past a tile, odd K: stores through shared memory
+                                   (513, 264, 512), (2000, 1030, 97), (64, 4096, 1024)])
+@pytest.mark.parametrize("special", [False, True])
+def test_weight_grad_fp32_split(C, m, k, n, special):
+    """The float32 gradient on the tensor cores: within the float32 summation bound of the float64 gradient, and rows
+    with infinities, NaN or values whose products overflow as the float32 chain gives them."""
+    rng = np.random.default_rng(m + k + n)
+    dy = (rng.standard_normal((m, n)) * 10.0 ** rng.uniform(-8, 2, (m, 1))).astype(F32)   # rows of very different scale
+    x = rng.standard_normal((k, n)).astype(F32)
+    x[:, 1] *= 1e6
+    if special:
+        dy[m - 1, n - 1], dy[3, 0], x[k - 1, 2], x[5, 7], dy[7, 4], x[9, 4] = np.inf, np.nan, -np.inf, 3e38, 1e30, -1e30
+    ws = _ws(C, m, k, n)
+    g = torch.full((m, k), float("nan"), device="cuda")
+    C.launch_count(reset=True)
+    C.weight_grad_dense(_dev(dy), _dev(x), g, ws, precision=0)
+    assert C.launch_count() == 2   # the split and the GEMM
+    got = g.cpu().numpy().astype(np.float64)
+    assert ws.status()[0] == 0
+    rows, cols = np.arange(m), np.arange(k)
+    if special:
+        rows, cols = np.setdiff1d(rows, [3, 7, m - 1]), np.setdiff1d(cols, [5, 9, k - 1])
+        assert np.isnan(got[3]).all()
+        with np.errstate(all="ignore"):
+            assert (got[m - 1, cols] == np.inf * np.sign(x[cols, n - 1])).all()
+            assert (got[rows, k - 1] == -np.inf * np.sign(dy[rows, 2])).all()
+            assert got[7, 9] == -np.inf   # 1e30 * -1e30
+    sub = np.ix_(rows, cols)
+    ref = dy.astype(np.float64)[rows] @ x.astype(np.float64)[cols].T
+    bound = np.abs(dy.astype(np.float64))[rows] @ np.abs(x.astype(np.float64))[cols].T
+    assert_close(got[sub], ref, bound, n, rtol=0, atol=0, what="fp32 split gradient")
+
+
 @pytest.mark.parametrize("m,k,n,density,zipf", [(300, 784, 64, 0.1, False), (100, 300, 256, 0.09, True),
                                                 (20, 25, 9000, 0.3, False), (50, 40, 1, 0.5, False),
                                                 (33, 17, 5, 0.0, False),
