@@ -31,13 +31,14 @@
 //
 // What bounds it: six bf16 products per multiply-add; 4096 x 4096 x 256 is
 // 51.5 GFLOP of MMA, 27 us at the measured bf16 rate, and 3.4 waves of tiles
-// run as 4. Measured (GB300, inputs in L2): 4096 x 4096 x 250 57.6 us (the
-// CUDA-core kernel 381), 4096 x 9216 x 256 107 us (830), 4096 x 4096 x 1024
-// 179 us (1464), 1000 x 4096 x 256 19 us (110). The MMAs alone take 0.91 us
-// per chunk and wave, with the operand loads and the reading back 1.15; a
+// run as 4. Measured (GB300, inputs in L2): 4096 x 4096 x 250 49 us (the
+// CUDA-core kernel 381), 4096 x 9216 x 256 91 us (830), 4096 x 4096 x 1024
+// 145 us (1464), 1000 x 4096 x 256 18 us (110). The MMAs alone take 0.91 us
+// per chunk and wave, with the operand loads and the reading back 1.0; a
 // wave's stores, which the next tile's first two chunks hide in part, 2-3 us.
 // 64-byte operand rows (stages of 32 columns) ran 11% slower than 128-byte
-// ones, eight reading warps with 128 sums each (spilling) 10%.
+// ones, eight reading warps with 128 sums each (spilling) 10%, arrivals with
+// .release.cluster 17-24%.
 #include "tc_pair.cuh"
 
 namespace csrt {
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
                     const int halves = imin(2, num_ch - 2 * kb);
                     for (int hf = 0; hf < halves; ++hf, ++ch) {
                         const int b = ch & 1;
-                        if (!mbar_wait_pair(acce + b, ((ch >> 1) & 1) ^ 1, &s_abort)) break;
+                        if (!mbar_wait_or_abort(acce + b, ((ch >> 1) & 1) ^ 1, &s_abort)) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t d = tmem + (uint32_t)(b * 256);
                         // planes of (dY, X): the small products first
@@ -374,7 +375,7 @@ int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_
     // GEMM within 15% over 64..4096 x 64..9216 x 32..1024, the CUDA-core
     // kernel, a latency per column or its 22 TFLOP/s, likewise).
     const double waves = (double)ceil_div(tiles, pairs), chunks = (double)ceil_div(n, kGsChunk);
-    const double t_split = 9.5 + waves * (2.8 + 1.15 * chunks);
+    const double t_split = 9.5 + waves * (2.5 + 1.0 * chunks);
     const double t_fma = imax(2.6 + 0.1 * imin(n, 512), 2.0 * m * k * n / 22e6);
     if (t_split > t_fma) return CSRT_OK;
     const int32_t ld = (int32_t)gs_ld(n);

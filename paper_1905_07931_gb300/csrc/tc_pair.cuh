@@ -33,26 +33,12 @@ __device__ __forceinline__ uint32_t map_to_rank(const void *p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
     return r;
 }
+// Arrives on a barrier of either CTA. (With .release.cluster the arrival waits
+// for every load the thread has in flight, over 1000 clocks for a prefetch;
+// what it has to order here is shared memory behind fence.proxy.async and
+// tensor memory behind tcgen05.wait and fence.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// mbar_wait_or_abort for a barrier that threads of the other CTA arrive on.
-__device__ __forceinline__ bool mbar_wait_pair(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
-    const uint32_t addr = smem_u32(bar);
-    for (unsigned i = 0; i < kTcWaitLimit; ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(addr), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if ((i & 63) == 63 && *abort_flag) return false;
-        if (i > 64) __nanosleep(32);
-    }
-    *abort_flag = 1;
-    return false;
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // 2-D TMA load into this CTA's shared memory, completing on a barrier given
 // by its shared::cluster address (the leader's).
