@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "spmm_tc.cuh"
 
 namespace csrt {
 
@@ -54,6 +55,8 @@ int csrt_workspace_bytes(int32_t rows, int32_t cols, int32_t max_n, size_t *byte
     size_t t = transpose_scratch_bytes(rows, cols);
     if (t > need) need = t;
     t = spmm_scratch_bytes(max_n);
+    if (t > need) need = t;
+    t = spmm_tc_scratch_bytes(rows, cols, max_n);
     if (t > need) need = t;
     t = sddmm_scratch_bytes(elems, max_n);
     if (t > need) need = t;

@@ -20,10 +20,12 @@
 // the workspace, or by a fix-up kernel), so the result is deterministic and
 // no float atomics are used. Narrow products (n <= 16 floats per vector width) put a
 // group of G < 32 lanes on each nonzero instead (spmm_group_kernel), and the
-// SDDMM uses the same grouped layout.
+// SDDMM uses the same grouped layout. Wide products of dense enough matrices
+// go to the tensor cores (spmm_tc.cu).
 #include <mutex>
 
 #include "common.cuh"
+#include "spmm_tc.cuh"
 
 namespace csrt {
 
@@ -92,6 +94,11 @@ struct SpmmArgs {
     int32_t relu;
     const float *mask;
     WsHeader *hdr;    // status word for a bounded wait that gives up (null: not reported)
+};
+// The wide kernel's: a tensor-core kernel follows for a matrix of tc.nnz_min
+// entries or more (0: none).
+struct SpmmWideArgs : SpmmArgs {
+    SpmmTcPrep tc;
 };
 
 // The epilogue of one row segment held by a lane (VW floats at column c).
@@ -227,16 +234,25 @@ __device__ __forceinline__ void spmm_complete_shared_rows(const SpmmArgs &a, int
 }
 
 template <int VW, int NV>
-__global__ void __launch_bounds__(kSpThreads, 3) spmm_merge_kernel(SpmmArgs a) {
+__global__ void __launch_bounds__(kSpThreads, VW * NV <= 2 ? 4 : 3) spmm_merge_kernel(SpmmWideArgs a) {
     pdl_enter();
     constexpr int TN = 32 * VW * NV;
     constexpr int kStride = 32 * VW;
     const int lane = threadIdx.x & 31;
+    const int64_t nnz = __ldg(a.row_ptr + a.rows);
+    if (a.tc.nnz_min > 0) {
+        // one wave of blocks: as each SM runs out of them, the next kernel's
+        // set up there (or are ready to leave at once)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+    if (a.tc.nnz_min > 0 && nnz >= a.tc.nnz_min) {
+        spmm_tc_prep(a.tc, a.row_ptr, a.col, a.val, a.rows, a.x, a.n);
+        return;
+    }
     const int64_t gw = ((int64_t)blockIdx.x * kSpThreads + threadIdx.x) >> 5;
     if (gw >= (int64_t)a.units * a.n_tiles) return;
     const int u = (int)(gw % a.units);
     const int t = (int)(gw / a.units);
-    const int64_t nnz = __ldg(a.row_ptr + a.rows);
     const int64_t items = (int64_t)a.rows + nnz;
     const int64_t per = ceil_div<int64_t>(items, a.units);
     const int64_t d0 = min((int64_t)u * per, items), d1 = min(d0 + per, items);
@@ -612,41 +628,45 @@ size_t spmm_scratch_bytes(int32_t max_n) {
 // Launches the product kernel of shape sh (and, for rows cut by units when
 // a.cnt is null, the fix-up kernel); returns the number of launches, or -1
 // for a shape without a kernel.
-static int spmm_dispatch(const SpmmShape &sh, const SpmmArgs &a, cudaStream_t s) {
+static int spmm_dispatch(const SpmmShape &sh, const SpmmArgs &args, const SpmmTcPrep &tc, cudaStream_t s) {
     const int64_t threads = (int64_t)sh.units * sh.n_tiles * 32;
     const unsigned grid = (unsigned)ceil_div<int64_t>(threads, kSpThreads);
-    const bool fix = sh.units > 1 && a.cnt == nullptr;
+    const bool fix = sh.units > 1 && args.cnt == nullptr;
+    SpmmWideArgs wide;
+    static_cast<SpmmArgs &>(wide) = args;
+    wide.tc = tc;
+    const size_t prep_smem = tc.nnz_min > 0 ? (size_t)(tc.chunks + 1) * 17 * sizeof(int32_t) : 0;
     const unsigned fg = (unsigned)ceil_div<int64_t>(threads, 256);
-#define CSRT_SPMM_CASE(VW, NV, G, KERNEL)                                                   \
+#define CSRT_SPMM_CASE(VW, NV, G, KERNEL, ARGS)                                             \
     if (sh.vw == VW && sh.nv == NV && sh.g == G) {                                          \
-        launch_pdl(KERNEL, dim3(grid), dim3(kSpThreads), G < 32 ? (size_t)kNarrowSmem : 0, s, a);           \
-        if (fix) launch_pdl(spmm_fixup_kernel<G * VW * NV>, dim3(fg), dim3(256), 0, s, a); \
+        launch_pdl(KERNEL, dim3(grid), dim3(kSpThreads), G < 32 ? (size_t)kNarrowSmem : prep_smem, s, ARGS); \
+        if (fix) launch_pdl(spmm_fixup_kernel<G * VW * NV>, dim3(fg), dim3(256), 0, s, args); \
         return fix ? 2 : 1;                                                                 \
     }
-    CSRT_SPMM_CASE(4, 2, 32, (spmm_merge_kernel<4, 2>))
-    CSRT_SPMM_CASE(4, 1, 32, (spmm_merge_kernel<4, 1>))
-    CSRT_SPMM_CASE(2, 1, 32, (spmm_merge_kernel<2, 1>))
-    CSRT_SPMM_CASE(1, 1, 32, (spmm_merge_kernel<1, 1>))
-    CSRT_SPMM_CASE(4, 1, 1, (spmm_group_kernel<4, 1>))
-    CSRT_SPMM_CASE(4, 1, 2, (spmm_group_kernel<4, 2>))
-    CSRT_SPMM_CASE(4, 1, 4, (spmm_group_kernel<4, 4>))
-    CSRT_SPMM_CASE(4, 1, 8, (spmm_group_kernel<4, 8>))
-    CSRT_SPMM_CASE(4, 1, 16, (spmm_group_kernel<4, 16>))
-    CSRT_SPMM_CASE(2, 1, 1, (spmm_group_kernel<2, 1>))
-    CSRT_SPMM_CASE(2, 1, 2, (spmm_group_kernel<2, 2>))
-    CSRT_SPMM_CASE(2, 1, 4, (spmm_group_kernel<2, 4>))
-    CSRT_SPMM_CASE(2, 1, 8, (spmm_group_kernel<2, 8>))
-    CSRT_SPMM_CASE(2, 1, 16, (spmm_group_kernel<2, 16>))
-    CSRT_SPMM_CASE(1, 1, 1, (spmm_group_kernel<1, 1>))
-    CSRT_SPMM_CASE(1, 1, 2, (spmm_group_kernel<1, 2>))
-    CSRT_SPMM_CASE(1, 1, 4, (spmm_group_kernel<1, 4>))
-    CSRT_SPMM_CASE(1, 1, 8, (spmm_group_kernel<1, 8>))
-    CSRT_SPMM_CASE(1, 1, 16, (spmm_group_kernel<1, 16>))
+    CSRT_SPMM_CASE(4, 2, 32, (spmm_merge_kernel<4, 2>), wide)
+    CSRT_SPMM_CASE(4, 1, 32, (spmm_merge_kernel<4, 1>), wide)
+    CSRT_SPMM_CASE(2, 1, 32, (spmm_merge_kernel<2, 1>), wide)
+    CSRT_SPMM_CASE(1, 1, 32, (spmm_merge_kernel<1, 1>), wide)
+    CSRT_SPMM_CASE(4, 1, 1, (spmm_group_kernel<4, 1>), args)
+    CSRT_SPMM_CASE(4, 1, 2, (spmm_group_kernel<4, 2>), args)
+    CSRT_SPMM_CASE(4, 1, 4, (spmm_group_kernel<4, 4>), args)
+    CSRT_SPMM_CASE(4, 1, 8, (spmm_group_kernel<4, 8>), args)
+    CSRT_SPMM_CASE(4, 1, 16, (spmm_group_kernel<4, 16>), args)
+    CSRT_SPMM_CASE(2, 1, 1, (spmm_group_kernel<2, 1>), args)
+    CSRT_SPMM_CASE(2, 1, 2, (spmm_group_kernel<2, 2>), args)
+    CSRT_SPMM_CASE(2, 1, 4, (spmm_group_kernel<2, 4>), args)
+    CSRT_SPMM_CASE(2, 1, 8, (spmm_group_kernel<2, 8>), args)
+    CSRT_SPMM_CASE(2, 1, 16, (spmm_group_kernel<2, 16>), args)
+    CSRT_SPMM_CASE(1, 1, 1, (spmm_group_kernel<1, 1>), args)
+    CSRT_SPMM_CASE(1, 1, 2, (spmm_group_kernel<1, 2>), args)
+    CSRT_SPMM_CASE(1, 1, 4, (spmm_group_kernel<1, 4>), args)
+    CSRT_SPMM_CASE(1, 1, 8, (spmm_group_kernel<1, 8>), args)
+    CSRT_SPMM_CASE(1, 1, 16, (spmm_group_kernel<1, 16>), args)
 #undef CSRT_SPMM_CASE
     return -1;
 }
 
-static int spmm_launch(const int32_t *row_ptr, const int32_t *col, const float *val, int32_t rows,
+static int spmm_launch(const int32_t *row_ptr, const int32_t *col, const float *val, int32_t rows, int32_t k,
                        int64_t capacity, const float *x, int32_t n, float *y, void *ws, size_t ws_bytes,
                        cudaStream_t s, const float *bias = nullptr, int32_t relu = 0, const float *mask = nullptr) {
     if (rows == 0 || n == 0) return CSRT_OK;
@@ -684,10 +704,19 @@ static int spmm_launch(const int32_t *row_ptr, const int32_t *col, const float *
         // us at n = 1, 1-2 us at n = 8 and 32, on 4096 x 4096 at 50%)
         if (sh.g == 32 && (int64_t)sh.units * sh.n_tiles <= (int64_t)kWsCounterInts) a.cnt = ws_counters(ws);
     }
-    const int launched = spmm_dispatch(sh, a, s);
+    SpmmTcPlan plan;
+    plan.prep.nnz_min = 0;
+    if (sh.g == 32 && (sh.units == 1 || a.cnt != nullptr)) {
+        // the sparse kernel's time per entry and n-tile (measured, 4096 x 4096)
+        const double t_tile = sh.nv == 2 ? 4.5e-5 : sh.vw == 4 ? 2.6e-5 : sh.vw == 2 ? 1.8e-5 : 1.7e-5;
+        spmm_tc_plan(rows, k, n, capacity, x, ws, ws_bytes, sh.units, t_tile * sh.n_tiles, &plan);
+    }
+    const int launched = spmm_dispatch(sh, a, plan.prep, s);
     CSRT_ARG(launched > 0, "spmm: no kernel for shape vw=%d nv=%d g=%d", sh.vw, sh.nv, sh.g);
     count_launch(launched);
-    return check_launch("spmm_merge_kernel");
+    const int rc = check_launch("spmm_merge_kernel");
+    if (rc || plan.prep.nnz_min == 0) return rc;
+    return spmm_tc_launch(plan, row_ptr, col, val, rows, x, n, y, bias, relu, mask, ws, s);
 }
 
 // Column-index ring of the narrow SDDMM: chunks of kSdChunk entries copied
@@ -975,7 +1004,7 @@ int spmm_fwd(const csrt_csr *w, const float *x, int32_t n, float *y, void *ws, s
     if (rc) return rc;
     CSRT_ARG(n >= 0, "n < 0");
     CSRT_ARG((x && y) || n == 0 || w->rows == 0, "X or Y is NULL");
-    return spmm_launch(w->row_ptr, w->col_idx, w->val, w->rows, w->capacity, x, n, y, ws, ws_bytes,
+    return spmm_launch(w->row_ptr, w->col_idx, w->val, w->rows, w->cols, w->capacity, x, n, y, ws, ws_bytes,
                        as_stream(stream));
 }
 
@@ -986,7 +1015,7 @@ int spmm_bwd_t(const csrt_csr *w, const float *dy, int32_t n, float *dx, void *w
     CSRT_ARG(w->t_row_ptr && w->t_col_idx && w->t_val, "transposed arrays not set");
     CSRT_ARG(n >= 0, "n < 0");
     CSRT_ARG((dy && dx) || n == 0 || w->cols == 0, "dY or dX is NULL");
-    return spmm_launch(w->t_row_ptr, w->t_col_idx, w->t_val, w->cols, w->capacity, dy, n, dx, ws, ws_bytes,
+    return spmm_launch(w->t_row_ptr, w->t_col_idx, w->t_val, w->cols, w->rows, w->capacity, dy, n, dx, ws, ws_bytes,
                        as_stream(stream));
 }
 
@@ -996,7 +1025,7 @@ int spmm_fwd_bias_act(const csrt_csr *w, const float *x, int32_t n, const float 
     if (rc) return rc;
     CSRT_ARG(n >= 0, "n < 0");
     CSRT_ARG((x && y) || n == 0 || w->rows == 0, "X or Y is NULL");
-    return spmm_launch(w->row_ptr, w->col_idx, w->val, w->rows, w->capacity, x, n, y, ws, ws_bytes,
+    return spmm_launch(w->row_ptr, w->col_idx, w->val, w->rows, w->cols, w->capacity, x, n, y, ws, ws_bytes,
                        as_stream(stream), bias, relu ? 1 : 0, nullptr);
 }
 
@@ -1007,7 +1036,7 @@ int spmm_bwd_t_relu(const csrt_csr *w, const float *dy, int32_t n, const float *
     CSRT_ARG(w->t_row_ptr && w->t_col_idx && w->t_val, "transposed arrays not set");
     CSRT_ARG(n >= 0, "n < 0");
     CSRT_ARG((dy && dx && y_below) || n == 0 || w->cols == 0, "dY, dX or the mask is NULL");
-    return spmm_launch(w->t_row_ptr, w->t_col_idx, w->t_val, w->cols, w->capacity, dy, n, dx, ws, ws_bytes,
+    return spmm_launch(w->t_row_ptr, w->t_col_idx, w->t_val, w->cols, w->rows, w->capacity, dy, n, dx, ws, ws_bytes,
                        as_stream(stream), nullptr, 0, y_below);
 }
 
@@ -1217,11 +1246,13 @@ extern "C" int spmm_fwd_noalloc(const csrt_csr *w, const float *x, int32_t n, fl
     a.carry = na->carry;
     a.carry_row = na->carry_row;
     a.cnt = nullptr;   // shared rows are completed by the fix-up kernel
+    SpmmTcPrep none;
+    none.nnz_min = 0;  // no workspace for the tensor-core path
     a.bias = nullptr;
     a.relu = 0;
     a.mask = nullptr;
     a.hdr = na->status;   // a bounded wait that gives up sets CSRT_DEV_TIMEOUT here
-    const int launched = spmm_dispatch(sh, a, as_stream(stream));
+    const int launched = spmm_dispatch(sh, a, none, as_stream(stream));
     CSRT_ARG(launched > 0, "spmm_fwd_noalloc: no kernel for shape vw=%d nv=%d g=%d", sh.vw, sh.nv, sh.g);
     count_launch(launched);
     return check_launch("spmm_fwd_noalloc");

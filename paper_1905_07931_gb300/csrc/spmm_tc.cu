@@ -1,0 +1,622 @@
+// Sparse x dense products on the tensor cores: Y = W X for a CSR matrix dense
+// enough that gathering a row of X per stored entry (n floats from L2 each)
+// costs more than multiplying the zeros.
+//
+// The product runs as a GEMM over all of W's columns in float32 accuracy.
+// Every factor is split into two fp16 parts, v = 2^s (hi + 2^-11 lo), with s
+// such that the largest magnitude that shares it lies in [2^14, 2^15): one s
+// per row of W, one per 64 features (rows) and 64 columns of X. hi and lo hold
+// 22 to 23 bits of every value down to 2^-29 of that largest one. Three products are taken,
+// hi lo' + lo hi' first and then hi hi' on top of them (the accumulator's
+// scale-input-d brings the first two down by 2^-11); lo lo' is below 2^-22.
+// tcgen05.mma truncates when it adds into its accumulator, so the sum of each
+// 64-column chunk of the reduction (four steps of hi hi') is read back and
+// added to float32 register sums, scaled by the chunk's power of two, with
+// round to nearest. Measured error against 64 bits: 1.2e-7 to 1.7e-7 where
+// the float32 chain of the sparse kernel has 1.6e-7 to 5.5e-7 (rows of 150 to
+// 2000 entries); layers whose rows hold fewer than 160 entries on average
+// keep the sparse kernel, whose short chains are more exact.
+//
+// W never exists densely in memory: the first kernel (spmm_tc.cuh) sorts its
+// split entries by groups of 16 rows and chunks of 64 columns, and eight warps
+// of each CTA put a chunk's entries into the cleared shared-memory operand of
+// the MMA (6 bytes per entry instead of 4 per element: written out as dense
+// planes, a layer at 5% took 52 us instead of 48, at 50% 83 instead of 96).
+//
+// Work: (256-row tile, kN columns of X) x 64-column chunks, cut into one
+// contiguous range per CTA pair. A pair whose range covers part of a tile's
+// chunks leaves a partial sum; the tile's pairs then share its columns and
+// add the parts up in pair order (st_share). Where there are enough tiles for
+// the GPU no tile is cut.
+//
+// Measured (GB300; the sparse kernel's time in brackets), rows x inner x n:
+// 4096 x 4096 x 256 at 20% 61 us (160), at 50% 96 (385), x 1024 at 5% 107
+// (170), at 50% 177 (1520), x 255 at 5% 51 (125); 4096 x 9216 x 256 at 5% 79
+// (99). At 4096 x 4096 x 256 and 5%: 10 us for the first kernel, 3 until the
+// first chunk's MMAs, 1.25 to 1.4 us per chunk (14 per pair; the MMAs alone
+// 1.0, slowed by the reading back and the expanding warps' stores, which use
+// the same tensor and shared memory), 10 for the partial sums (20 MB written
+// and read in L2).
+//
+// Values a factor can't take here (2^50 and more, infinities, NaN) turn the
+// scale of their row or chunk into NaN, which ends as a NaN in the sums they
+// touch; such entries of Y are computed again from the CSR row.
+#include "spmm_tc.cuh"
+#include "tc_pair.cuh"
+
+namespace csrt {
+
+constexpr int kStChunk = kTcChunk;
+// Warps: 0 TMA, 1 MMA (2 and 3 idle), eight that expand W (a group of 16 rows
+// each), sixteen that add up and write; registers within the launch's 896 x 72.
+constexpr int kStExpandWarps = 8, kStEpiWarps = 16;
+constexpr int kStThreads = 32 * (4 + kStExpandWarps + kStEpiWarps);
+constexpr int kStProdRegs = 32, kStExpandRegs = 40, kStEpiRegs = 96;
+static_assert(128 * kStProdRegs + 32 * (kStExpandWarps * kStExpandRegs + kStEpiWarps * kStEpiRegs) <= kStThreads * 72,
+              "register split");
+constexpr int kStASlice = 128 * kStChunk * 2;
+template <int kN> __host__ __device__ constexpr int st_bslice() { return kN / 2 * kStChunk * 2; }
+template <int kN> __host__ __device__ constexpr int st_stage() { return 2 * (kStASlice + st_bslice<kN>()); }
+template <int kN> __host__ __device__ constexpr int st_stages() { return kN == 256 ? 3 : 4; }
+template <int kN> __host__ __device__ constexpr int st_smem() { return st_stages<kN>() * st_stage<kN>() + 256 + 1024; }
+static_assert(st_smem<256>() <= 232448 && st_smem<128>() <= 232448, "shared memory per block");
+
+struct StArgs {
+    const int32_t *row_ptr, *col;
+    const float *val;
+    int32_t rows, k, n;
+    const uint32_t *parts;
+    const uint16_t *place;
+    const int32_t *start;
+    const float *x, *wscale, *xscale;
+    float *y, *partial;
+    uint32_t *cnt;
+    const float *bias, *mask;
+    int32_t relu;
+    int64_t nnz_min;
+    int32_t tiles_n, tiles, chunks, pairs;
+    int32_t whole;   // pairs take whole tiles
+    WsHeader *hdr;
+};
+
+__device__ __forceinline__ int32_t ld_row_end(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void mma_f16_pair_down11(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p, 11;\n}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc)
+        : "memory");
+}
+
+// Entry (row, c) of the product from the CSR row, as the sparse kernel adds it.
+static __device__ __noinline__ float st_entry(const StArgs &a, int64_t row, int64_t c) {
+    float sum = 0.f;
+    for (int32_t k = a.row_ptr[row]; k < a.row_ptr[row + 1]; ++k)
+        sum = fmaf(__ldg(a.val + k), __ldg(a.x + (int64_t)__ldg(a.col + k) * a.n + c), sum);
+    return sum;
+}
+
+__device__ __forceinline__ float st_finish(const StArgs &a, int64_t row, int64_t c, float v) {
+    if (a.bias) v = __fadd_rn(v, __ldg(a.bias + row));
+    if (a.relu) v = fmaxf(v, 0.f);
+    if (a.mask && !(__ldg(a.mask + row * a.n + c) > 0.f)) v = 0.f;
+    return v;
+}
+
+// First unit of pair p, and the pair that unit u belongs to.
+__host__ __device__ inline int64_t st_first(int64_t units, int pairs, int p) { return units * p / pairs; }
+__host__ __device__ inline int st_pair_of(int64_t units, int pairs, int64_t u) {
+    return (int)(((u + 1) * pairs - 1) / units);
+}
+// The partial sum a pair leaves of a tile it shares: two slots per pair (the
+// beginning of a tile, or a later part) and CTA, 128 x kN floats each.
+template <int kN>
+__device__ __forceinline__ float *st_slot(const StArgs &a, int pair, bool beginning, uint32_t rank) {
+    return a.partial + ((int64_t)(pair * 2 + (beginning ? 1 : 0)) * 2 + rank) * 128 * kN;
+}
+
+__device__ __forceinline__ float st_row_scale(const StArgs &a, int tile, uint32_t rank, int q) {
+    const int64_t row = (int64_t)(tile / a.tiles_n) * 256 + rank * 128 + q * 32 + (threadIdx.x & 31);
+    return row < a.rows ? __ldg(a.wscale + row) : 0.f;
+}
+// Eight columns (c .. c + 7 of the tile) of row 32q + lane of the CTA's half
+// of a tile: W's row scale, the epilogue, Y.
+template <int kN>
+__device__ __forceinline__ void st_write(const StArgs &a, int tile, uint32_t rank, int q, int c, const float *sum,
+                                         float wsc) {
+    const int64_t row = (int64_t)(tile / a.tiles_n) * 256 + rank * 128 + q * 32 + (threadIdx.x & 31);
+    const int64_t col = (int64_t)(tile % a.tiles_n) * kN + c;
+    if (row >= a.rows || col >= a.n) return;
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = sum[i] * wsc;
+    if (isnan(v[0])) {
+        for (int i = 0; i < 8 && col + i < a.n; ++i)
+            a.y[row * a.n + col + i] = st_finish(a, row, col + i, st_entry(a, row, col + i));
+        return;
+    }
+    if (a.bias || a.relu || a.mask) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (col + i < a.n) v[i] = st_finish(a, row, col + i, v[i]);
+    }
+    float *dst = a.y + row * a.n + col;
+    if (a.n % 8 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 31) == 0) {
+        st_global_f8(dst, v);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (col + i < a.n) dst[i] = v[i];
+    }
+}
+
+// Counting in at a cut tile. cnt[0]: the parts that are there (bits 0-7) and
+// the shares whose pairs gave up waiting (from bit 8); cnt[1]: the pairs that
+// are through, the last of which zeroes both.
+constexpr uint32_t kStPartsMask = 0xff;
+
+// One pair's part in adding up a cut tile; `seen` is what cnt[0] was when it
+// counted in.
+template <int kN>
+__device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, int tile, uint32_t rank, int q, int h,
+                                      int tid, uint32_t seen, volatile uint32_t *state) {
+    constexpr int kUnits = kN / 32;   // eights of an epilogue warp's columns
+    const int64_t t0 = (int64_t)tile * a.chunks;
+    const int p0 = st_pair_of(units, a.pairs, t0), parts = st_pair_of(units, a.pairs, t0 + a.chunks - 1) - p0 + 1;
+    // (the pair that begins a tile has ended another, whose share it does)
+    const int shares = imin(parts - 1, kUnits), own = pair - p0 - 1;
+    uint32_t *cnt = a.cnt + 2 * (tile * 2 + (int)rank);
+    if (tid == 0) {
+        uint32_t todo = own >= 0 && own < shares ? 1u << own : 0u;
+        if ((int)(seen & kStPartsMask) == parts - 1) {
+            todo |= seen >> 8;   // the last to come: also the shares given up before
+            __threadfence();
+        } else if (todo) {
+            bool all = false;
+            for (int i = 0; i < 400; ++i) {
+                uint32_t now;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(cnt) : "memory");
+                if ((all = (int)(now & kStPartsMask) == parts)) break;
+                __nanosleep(20);
+            }
+            // gives up; whoever counts in last takes the share, unless it just has
+            if (!all && (int)(atomicOr(cnt, todo << 8) & kStPartsMask) != parts) todo = 0;
+            if (!all) __threadfence();
+        }
+        *state = todo;
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kStEpiWarps) : "memory");
+    uint32_t todo = *state;
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kStEpiWarps) : "memory");   // state is read
+    const float wsc = st_row_scale(a, tile, rank, q);
+    for (; todo; todo &= todo - 1) {
+        const int s = __ffs((int)todo) - 1;
+        for (int c = kUnits * s / shares; c < kUnits * (s + 1) / shares; ++c) {
+            // six parts' loads in flight (a tile rarely has more): the time here
+            // is that of the L2 round trips, 1 to 2 us each under this load
+            float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int p = 0; p < parts; p += 6) {
+                float x[6][8];
+#pragma unroll
+                for (int o = 0; o < 6; ++o)
+                    if (p + o < parts)
+                        ld_global_f8(st_slot<kN>(a, p0 + p + o, p + o == 0, rank) + (c * 32 * kStEpiWarps + tid) * 8, x[o]);
+#pragma unroll
+                for (int o = 0; o < 6; ++o)
+                    if (p + o < parts) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) v[i] += x[o][i];
+                    }
+            }
+            st_write<kN>(a, tile, rank, q, h * (kN / 4) + c * 8, v, wsc);
+        }
+    }
+    if (tid == 0 && (int)atomicAdd(cnt + 1, 1u) == parts - 1) cnt[0] = cnt[1] = 0;
+}
+
+template <int kN>
+__global__ void __launch_bounds__(kStThreads, 1)
+    spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, StArgs a) {
+    // The first kernel's blocks have all passed their own wait when this kernel
+    // starts, so the row pointers (which it does not write) are complete.
+    if (ld_row_end(a.row_ptr + a.rows) < a.nnz_min) {
+        pdl_enter();   // (whoever waits for this kernel waits for the one before, too)
+        return;        // the sparse kernel before this one does the product
+    }
+    constexpr int kStages = st_stages<kN>(), kStage = st_stage<kN>(), kBSlice = st_bslice<kN>();
+    constexpr int kCols = kN / 4;   // columns of an epilogue warp
+    constexpr uint32_t kIdesc = idesc_f16(0, 256, kN);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStage);
+    uint64_t *empty = full + kStages;
+    uint64_t *accf = empty + kStages;
+    uint64_t *acce = accf + 2;
+    uint64_t *fin = acce + 2;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
+    __shared__ volatile int s_abort;
+    __shared__ volatile uint32_t s_state;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int pair = blockIdx.x >> 1;
+    const int64_t units = (int64_t)a.tiles * a.chunks;
+    const int64_t u_begin = a.whole ? st_first(a.tiles, a.pairs, pair) * a.chunks : st_first(units, a.pairs, pair);
+    const int64_t u_end = a.whole ? st_first(a.tiles, a.pairs, pair + 1) * a.chunks : st_first(units, a.pairs, pair + 1);
+
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(full + s, 1 + 2 * kStExpandWarps);
+            mbar_init(empty + s, 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(accf + b, 1);
+            mbar_init(acce + b, 2 * kStEpiWarps);
+        }
+        mbar_init(fin, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_x)) : "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(2 * kN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync_all();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+    pdl_enter();   // the operands are complete from here on
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kStProdRegs));
+        if (warp == 0 && lane == 0) {
+            int it = 0;
+            int tile = (int)(u_begin / a.chunks), ch = (int)(u_begin % a.chunks);
+            for (int64_t u = u_begin; u < u_end && !s_abort; ++u, ++it) {
+                const int c0 = (tile % a.tiles_n) * kN + (int)rank * (kN / 2);
+                const int s = it % kStages;
+                if (!mbar_wait_or_abort(empty + s, ((it / kStages) & 1) ^ 1, &s_abort)) break;
+                if (rank == 0) mbar_expect_tx(full + s, 4 * kBSlice);
+                const uint32_t bar = map_to_rank(full + s, 0);
+                uint8_t *st = smem + s * kStage + 2 * kStASlice;
+                tma_load_2d_pair(st, &map_x, ch * kStChunk, c0, bar);
+                tma_load_2d_pair(st + kBSlice, &map_x, ch * kStChunk, a.n + c0, bar);
+                if (++ch == a.chunks) {
+                    ch = 0;
+                    ++tile;
+                }
+            }
+            // every load of both CTAs must land before the pair may exit
+            if (rank == 0)
+                for (int i = imax(0, it - kStages); i < it; ++i) mbar_wait(full + i % kStages, (i / kStages) & 1);
+        } else if (warp == 1 && lane == 0 && rank == 0) {
+            int it = 0;
+            for (int64_t u = u_begin; u < u_end && !s_abort; ++u, ++it) {
+                const int s = it % kStages, b = it & 1;
+                if (!mbar_wait_or_abort(acce + b, ((it >> 1) & 1) ^ 1, &s_abort)) break;
+                if (!mbar_wait_or_abort(full + s, (it / kStages) & 1, &s_abort)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint8_t *ah = smem + s * kStage, *al = ah + kStASlice;
+                const uint8_t *bh = ah + 2 * kStASlice, *bl = bh + kBSlice;
+                const uint32_t d = tmem + (uint32_t)(b * kN);
+#pragma unroll
+                for (int k = 0; k < kStChunk / 16; ++k)
+                    mma_f16_pair(d, smem_desc_sw128(ah + k * 32), smem_desc_sw128(bl + k * 32), kIdesc, k > 0);
+#pragma unroll
+                for (int k = 0; k < kStChunk / 16; ++k)
+                    mma_f16_pair(d, smem_desc_sw128(al + k * 32), smem_desc_sw128(bh + k * 32), kIdesc, 1u);
+                mma_f16_pair_down11(d, smem_desc_sw128(ah), smem_desc_sw128(bh), kIdesc);
+#pragma unroll
+                for (int k = 1; k < kStChunk / 16; ++k)
+                    mma_f16_pair(d, smem_desc_sw128(ah + k * 32), smem_desc_sw128(bh + k * 32), kIdesc, 1u);
+                mma_commit_pair(empty + s);
+                mma_commit_pair(accf + b);
+            }
+            asm volatile(
+                "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(fin))
+                : "memory");
+            mbar_wait(fin, 0);
+        }
+    } else if (warp < 4 + kStExpandWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kStExpandRegs));
+        // An expanding warp: one group of 16 rows. Per chunk it clears their
+        // 128 bytes in both planes and puts the entries' parts at their
+        // places, 256 entries at a time. The next entries are asked for as
+        // soon as these are in place: their latency (1000 clocks under load)
+        // passes while the MMAs of the stages ahead run. The bounds of 31
+        // chunks lie in the lanes of one register.
+        const int e = warp - 4;
+        const int groups = (a.rows + kTcGroup - 1) / kTcGroup;
+        int tile = (int)(u_begin / a.chunks), ch = (int)(u_begin % a.chunks);
+        int32_t ends = 0;
+        int ch_ends = 0;   // lane l of `ends`: start[ch_ends + l]
+        auto load_ends = [&]() {
+            const int g = (tile / a.tiles_n) * 16 + (int)rank * 8 + e;
+            ch_ends = ch;
+            ends = g < groups ? __ldg(a.start + (int64_t)g * (a.chunks + 1) + imin(ch + lane, a.chunks)) : 0;
+        };
+        uint32_t part[8], place[8];
+        auto fetch = [&](int32_t i, int32_t hi) {
+#pragma unroll
+            for (int h = 0; h < 8; ++h) {
+                const bool on = i + h * 32 + lane < hi;
+                part[h] = on ? __ldg(a.parts + i + h * 32 + lane) : 0u;
+                place[h] = on ? __ldg(a.place + i + h * 32 + lane) : 0xffffu;
+            }
+        };
+        load_ends();
+        int32_t lo = __shfl_sync(0xffffffffu, ends, 0), hi = __shfl_sync(0xffffffffu, ends, 1);
+        fetch(lo, hi);
+        int it = 0;
+        for (int64_t u = u_begin; u < u_end; ++u, ++it) {
+            int32_t lo_n = 0, hi_n = 0;   // the next chunk's entries
+            if (u + 1 < u_end) {
+                if (++ch == a.chunks) {
+                    ch = 0;
+                    ++tile;
+                    load_ends();
+                } else if (ch - ch_ends == 31) {
+                    load_ends();
+                }
+                lo_n = __shfl_sync(0xffffffffu, ends, ch - ch_ends);
+                hi_n = __shfl_sync(0xffffffffu, ends, ch - ch_ends + 1);
+            }
+            const int s = it % kStages;
+            uint8_t *base = smem + s * kStage + e * (kTcGroup * 128);
+            if (!__all_sync(0xffffffffu, mbar_wait_or_abort(empty + s, ((it / kStages) & 1) ^ 1, &s_abort))) break;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                *reinterpret_cast<uint4 *>(base + i * 512 + lane * 16) = make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4 *>(base + kStASlice + i * 512 + lane * 16) = make_uint4(0, 0, 0, 0);
+            }
+            __syncwarp();
+            while (true) {
+#pragma unroll
+                for (int h = 0; h < 8; ++h)
+                    if (place[h] != 0xffffu) {
+                        *reinterpret_cast<uint16_t *>(base + place[h]) = (uint16_t)part[h];
+                        *reinterpret_cast<uint16_t *>(base + kStASlice + place[h]) = (uint16_t)(part[h] >> 16);
+                    }
+                lo += 256;
+                if (lo >= hi) break;
+                fetch(lo, hi);
+            }
+            fetch(lo_n, hi_n);
+            lo = lo_n;
+            hi = hi_n;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_to_rank(full + s, 0));
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kStEpiRegs));
+        const int q = warp & 3;             // TMEM lanes 32q ..
+        const int h = (warp - 4 - kStExpandWarps) >> 2;   // column quarter of the tile
+        const int tid = threadIdx.x - 32 * (4 + kStExpandWarps);
+        const uint32_t acce0 = map_to_rank(acce, 0), acce1 = map_to_rank(acce + 1, 0);
+        int it = 0, tile_e = -1, tile_b = -1;
+        uint32_t seen_e = 0, seen_b = 0;   // (thread 0)
+        bool ok = true;
+        for (int64_t u = u_begin; u < u_end;) {
+            const int tile = (int)(u / a.chunks), ch0 = (int)(u % a.chunks);
+            const int ch1 = (int)imin<int64_t>(a.chunks, ch0 + (u_end - u));
+            float acc[kCols];
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
+            const int nb = (a.n + kCols - 1) / kCols, xb = imin((tile % a.tiles_n) * 4 + h, nb - 1);
+            float sc = __ldg(a.xscale + ch0 * nb + xb);
+            for (int ch = ch0; ch < ch1; ++ch, ++it) {
+                const int b = it & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait_or_abort(accf + b, (it >> 1) & 1, &s_abort));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int c = 0; c < kCols; c += 16) {
+                    uint32_t r[16];
+                    tmem_ld_16cols(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kN + h * kCols + c), r);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) acc[c + i] = fmaf(__uint_as_float(r[i]), sc, acc[c + i]);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(b ? acce1 : acce0);
+                sc = __ldg(a.xscale + imin(ch + 1, a.chunks - 1) * nb + xb);
+            }
+            if (!ok) break;
+            u += ch1 - ch0;
+            if (ch0 == 0 && ch1 == a.chunks) {
+                const float wsc = st_row_scale(a, tile, rank, q);
+#pragma unroll
+                for (int c = 0; c < kCols; c += 8) st_write<kN>(a, tile, rank, q, h * kCols + c, acc + c, wsc);
+                continue;
+            }
+            // A partial sum: left in the workspace, counted in. (A pair's
+            // first range may end a tile, its last may begin one.)
+            const bool begins = ch0 == 0;
+            float *mine = st_slot<kN>(a, pair, begins, rank) + tid * 8;
+#pragma unroll
+            for (int c = 0; c < kCols; c += 8) st_global_f8(mine + c * (32 * kStEpiWarps), acc + c);
+            __threadfence();
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kStEpiWarps) : "memory");
+            if (tid == 0) {
+                const uint32_t seen = atomicAdd(a.cnt + 2 * (tile * 2 + (int)rank), 1u);
+                if (begins) seen_b = seen;
+                else seen_e = seen;
+            }
+            if (begins) tile_b = tile;
+            else tile_e = tile;
+        }
+        // The cut tiles: their pairs share the work of adding the partial
+        // sums (in pair order, so the result does not depend on who adds).
+        // All pairs finish at about the same time: each waits a moment (some
+        // 15 us at most) until a tile's parts are all there and takes its own
+        // share of the columns. One that has waited in vain leaves a note and
+        // goes; the last pair to count in does the shares of those, so
+        // nothing depends on all pairs being resident at once.
+        if (ok) {
+            if (tile_e >= 0) st_share<kN>(a, units, pair, tile_e, rank, q, h, tid, seen_e, &s_state);
+            if (tile_b >= 0) st_share<kN>(a, units, pair, tile_b, rank, q, h, tid, seen_b, &s_state);
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0 && s_abort) {
+        dev_flag(a.hdr, CSRT_DEV_TIMEOUT);
+        a.hdr->timeout_site = 12;
+    }
+    cluster_sync_all();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kN) : "memory");
+    }
+}
+
+static size_t st_align(size_t v) { return (v + 255) / 256 * 256; }
+static int32_t st_ld(int32_t k) { return (int32_t)ceil_div<int64_t>(k, 8) * 8; }
+static int st_max_pairs() { return imax(1, num_sms() / 2); }
+// Entries, planes, scales and partial sums of a rows x k matrix of at most
+// `capacity` entries and n columns.
+static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int64_t capacity, int n_tile) {
+    const int64_t chunks = ceil_div(k, kStChunk);
+    return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)4 * n * st_ld(k)) +
+           st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) + st_align((size_t)4 * rows) +
+           st_align((size_t)4 * chunks * ceil_div(n, n_tile / 4)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
+}
+constexpr int32_t kStMinRows = 256, kStMinK = 1024, kStMinN = 65;
+static bool st_shape_ok(int32_t rows, int32_t k) {
+    return rows >= kStMinRows && k >= kStMinK && k <= kTcMaxChunks * kStChunk;
+}
+
+size_t spmm_tc_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
+    if (max_n < kStMinN) return 0;
+    const bool fwd = st_shape_ok(rows, cols), bwd = st_shape_ok(cols, rows);
+    if (!fwd && !bwd) return 0;
+    const int64_t all = (int64_t)rows * cols;
+    const size_t f = fwd ? st_bytes(rows, cols, max_n, all, 256) : 0, b = bwd ? st_bytes(cols, rows, max_n, all, 256) : 0;
+    return imax(f, b) <= (size_t)1 << 30 ? imax(f, b) : 0;   // beyond a gigabyte: the sparse kernel alone
+}
+
+void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const float *x, void *ws, size_t ws_bytes,
+                  int32_t sparse_units, double t_entry, SpmmTcPlan *plan) {
+    plan->prep.nnz_min = 0;
+    if (!st_shape_ok(rows, k) || n < kStMinN || ws == nullptr || !device_is_sm10x()) return;
+    const int n_tile = n <= 128 ? 128 : 256;
+    capacity = imin<int64_t>(capacity, (int64_t)rows * k);
+    if (ws_bytes < kWsReservedBytes + st_bytes(rows, k, n, capacity, n_tile)) return;
+    const int chunks = ceil_div(k, kStChunk);
+    plan->n_tile = n_tile;
+    plan->tiles_n = ceil_div(n, n_tile);
+    plan->tiles = ceil_div(rows, 256) * plan->tiles_n;
+    if (4 * plan->tiles > (int)kWsCounterInts) return;
+    const int64_t units = (int64_t)plan->tiles * chunks;
+    // Whole tiles per pair where that costs no more than cutting them
+    // (microseconds; the partial sums take 4 us and 2.2 us for each eighth of
+    // a tile's columns that a pair has to add up).
+    const int max_pairs = st_max_pairs();
+    const double t_unit = n_tile == 256 ? 1.25 : 0.85;
+    const int cut_pairs = (int)imin<int64_t>(units, max_pairs);
+    const double whole = (double)ceil_div(plan->tiles, max_pairs) * chunks * t_unit;
+    const double cut = (double)ceil_div<int64_t>(units, cut_pairs) * t_unit + 4.0 +
+                       2.2 * ceil_div(n_tile / 32, imax(1, cut_pairs / plan->tiles));
+    plan->whole = whole <= cut;
+    plan->pairs = plan->whole ? ceil_div(plan->tiles, ceil_div(plan->tiles, max_pairs)) : cut_pairs;
+    // The number of entries from which this path is the faster one: both
+    // times are fits to measurements over 512..9216 rows and columns, 1% to
+    // 50% and 100 to 1024 columns of X (within 15%):
+    //   here    15 us (both operands, launches, first and last steps), the
+    //           chunks, 8.5e-6 us per entry (sorting and expanding it);
+    //   sparse  8.5 us and t_entry per entry.
+    // And the number from which it is the more exact one: a sum of the sparse
+    // kernel runs over a row, or over the part of it in one unit, and its
+    // error grows with that length (1.0e-7 at 50, 1.4e-7 at 110, 1.6e-7 at
+    // 200, 5.5e-7 at 2000), here it is 1.2e-7 to 1.4e-7 (1.7e-7 at 2000).
+    const double t_tc = 15.0 + imin(whole, cut);
+    if (t_entry <= 9e-6) return;
+    const int64_t nnz_min = imax<int64_t>(imax<int64_t>((int64_t)rows * 160, (int64_t)sparse_units * 128),
+                                          (int64_t)(1.05 * (t_tc - 8.5) / (t_entry - 8.5e-6)));
+    // Where the sparse kernel turns out to be the better one, the launch that
+    // follows it in vain costs 1.5 us (and the host 4): not where only the
+    // densest matrices would gain.
+    if (nnz_min > capacity || (double)nnz_min > 0.09 * rows * k) return;
+    char *p = ws_scratch(ws);
+    p = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(p) + 255) & ~uintptr_t(255));
+    auto take = [&](size_t bytes) {
+        char *at = p;
+        p += st_align(bytes);
+        return at;
+    };
+    plan->prep.parts = reinterpret_cast<uint32_t *>(take((size_t)4 * capacity));
+    plan->prep.place = reinterpret_cast<uint16_t *>(take((size_t)2 * capacity));
+    plan->prep.xp = reinterpret_cast<__half *>(take((size_t)4 * n * st_ld(k)));
+    plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)));
+    plan->prep.wscale = reinterpret_cast<float *>(take((size_t)4 * rows));
+    plan->prep.xscale = reinterpret_cast<float *>(take((size_t)4 * chunks * ceil_div(n, n_tile / 4)));
+    plan->partial = reinterpret_cast<float *>(p);
+    plan->cnt = ws_counters(ws);
+    plan->prep.k = k;
+    plan->prep.ld = st_ld(k);
+    plan->prep.chunks = chunks;
+    plan->prep.width = n_tile / 4;
+    plan->prep.vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    plan->prep.nnz_min = nnz_min;
+}
+
+int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t *col, const float *val, int32_t rows,
+                   const float *x, int32_t n, float *y, const float *bias, int32_t relu, const float *mask, void *ws,
+                   cudaStream_t s) {
+    CUtensorMap mx;
+    const int32_t k = plan.prep.k;
+    if (!make_map16(&mx, plan.prep.xp, false, (int64_t)2 * n, k, plan.prep.ld, plan.n_tile / 2, kStChunk))
+        return fail(CSRT_ERR_CUDA, "spmm: the tensor map of X's planes could not be made");
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    CSRT_CHECK_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        CSRT_CHECK_CUDA(cudaFuncSetAttribute(spmm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             st_smem<256>()));
+        CSRT_CHECK_CUDA(cudaFuncSetAttribute(spmm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             st_smem<128>()));
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    StArgs a;
+    a.row_ptr = row_ptr;
+    a.col = col;
+    a.val = val;
+    a.rows = rows;
+    a.k = k;
+    a.n = n;
+    a.parts = plan.prep.parts;
+    a.place = plan.prep.place;
+    a.start = plan.prep.start;
+    a.x = x;
+    a.wscale = plan.prep.wscale;
+    a.xscale = plan.prep.xscale;
+    a.y = y;
+    a.partial = plan.partial;
+    a.cnt = reinterpret_cast<uint32_t *>(plan.cnt);
+    a.bias = bias;
+    a.mask = mask;
+    a.relu = relu;
+    a.nnz_min = plan.prep.nnz_min;
+    a.tiles_n = plan.tiles_n;
+    a.tiles = plan.tiles;
+    a.chunks = plan.prep.chunks;
+    a.pairs = plan.pairs;
+    a.whole = plan.whole;
+    a.hdr = static_cast<WsHeader *>(ws);
+    const unsigned grid = (unsigned)(2 * plan.pairs);
+    if (plan.n_tile == 256) launch_pair(spmm_tc_kernel<256>, grid, kStThreads, st_smem<256>(), s, mx, a);
+    else launch_pair(spmm_tc_kernel<128>, grid, kStThreads, st_smem<128>(), s, mx, a);
+    count_launch();
+    return check_launch("spmm_tc_kernel");
+}
+
+}  // namespace csrt

@@ -100,6 +100,13 @@ __device__ __forceinline__ void st_global_f8(float *p, const float *v) {
                  : "memory");
 }
 
+__device__ __forceinline__ void ld_global_f8(const float *p, float (&v)[8]) {
+    asm volatile("ld.relaxed.gpu.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+
 // Row-major rows x cols matrix of 16-bit elements with row stride ld elements
 // (a multiple of 8): boxes of box_rows x 32 elements (64-byte swizzle) or x 64
 // (128-byte swizzle).

@@ -302,6 +302,92 @@ def test_spmm_is_deterministic(C, m, k, n):
     np.testing.assert_array_equal(ys[0].view(np.uint32), ys[2].view(np.uint32))
 
 
+# Shapes whose products take the tensor cores where the matrix is dense enough (as these are): column tiles of 128 and
+# 256, whole and shared tiles, ragged rows, inner columns and n (odd: no vector loads or stores), power-law rows, groups
+# with several hundred entries in a chunk.
+TC_CASES = [(777, 2500, 333, 0.12, True), (700, 4000, 255, 0.3, False), (1300, 5000, 99, 0.1, False),
+            (1025, 4000, 1024, 0.12, False), (4000, 4000, 1000, 0.06, False), (1030, 4160, 129, 0.99, False)]
+
+
+def _tc_case(C, m, k, n, density, zipf):
+    rng = np.random.default_rng(m + k + n)
+    a = _sparse(rng, m, k, density, zipf)
+    a *= (10.0 ** rng.uniform(-6, 2, (m, 1))).astype(F32)        # rows of very different scale
+    a[2, :] = 0.0
+    x = rng.standard_normal((k, n)).astype(F32) * (10.0 ** rng.uniform(-2, 2, (k, 1))).astype(F32)
+    ws = _ws(C, m, k, n)
+    return a, x, ws, _gpu_csr(C, a, ws, capacity=int((a != 0).sum()) + 7)
+
+
+@pytest.mark.parametrize("m,k,n,density,zipf", TC_CASES)
+def test_spmm_tensor_core_path(C, m, k, n, density, zipf):
+    """Forward with bias and ReLU, and transposed with the mask, against float64: within the float32 summation bound
+    plus the parts' representation (2^-23 per factor, 2^-22 for the product of the low parts left out)."""
+    a, x, ws, w = _tc_case(C, m, k, n, density, zipf)
+    rng = np.random.default_rng(1)
+    bias = rng.standard_normal(m).astype(F32)
+    dy, below = rng.standard_normal((m, n)).astype(F32), np.maximum(rng.standard_normal((k, n)), 0).astype(F32)
+    A, X, DY = (_dev(t).double() for t in (a, x, dy))
+    lens, tlens = (A != 0).sum(1, keepdim=True).double(), (A != 0).sum(0)[:, None].double()
+    u = 2.0 ** -24
+    y = torch.full((m, n), float("nan"), device="cuda")
+    C.launch_count(reset=True)
+    C.spmm_fwd(w, _dev(x), y, ws)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    ref, S = A @ X, A.abs() @ X.abs()
+    lim = (2.0 ** -21 + (lens + 64) * u) * S + u * ref.abs() + 1e-30
+    assert ((y.double() - ref).abs() <= lim).all()
+    y2 = torch.full((m, n), float("nan"), device="cuda")
+    C.spmm_fwd_bias_act(w, _dev(x), _dev(bias), True, y2, ws)
+    np.testing.assert_array_equal(y2.cpu().numpy(), np.maximum(y.cpu().numpy() + bias[:, None], 0))
+    dx = torch.full((k, n), float("nan"), device="cuda")
+    C.spmm_bwd_t_relu(w, _dev(dy), _dev(below), dx, ws)
+    ref, S = (A.T @ DY) * (_dev(below) > 0), A.abs().T @ DY.abs()
+    lim = (2.0 ** -21 + (tlens + 64) * u) * S + u * ref.abs() + 1e-30
+    assert ((dx.double() - ref).abs() <= lim).all()
+    assert ws.status()[0] == 0
+    # the counters of shared tiles are left zero: the same again
+    y3 = torch.full((m, n), float("nan"), device="cuda")
+    C.spmm_fwd(w, _dev(x), y3, ws)
+    np.testing.assert_array_equal(y3.cpu().numpy().view(np.uint32), y.cpu().numpy().view(np.uint32))
+
+
+@pytest.mark.parametrize("m,k,n,density,zipf", TC_CASES[:5:2])
+def test_spmm_tensor_core_path_special_values(C, m, k, n, density, zipf):
+    """Infinities, NaN and values whose products overflow, in X and in W: rows of Y that do not store them are as
+    without them, the others as the float32 sums over the stored entries give them."""
+    a, x, ws, w = _tc_case(C, m, k, n, density, zipf)
+    clean = torch.full((m, n), float("nan"), device="cuda")
+    C.spmm_fwd(w, _dev(x), clean, ws)
+    xs = x.copy()
+    xs[7, 3], xs[k - 1, n - 1], xs[70, 0], xs[71, 1] = np.inf, np.nan, 3e38, -1e30
+    r = int(np.flatnonzero((a != 0).sum(1) > 3)[5])
+    j = int(np.flatnonzero(a[r])[1])
+    a2 = a.copy()
+    a2[r, j] = -np.inf
+    w2 = _gpu_csr(C, a2, ws)
+    y = torch.full((m, n), float("nan"), device="cuda")
+    C.spmm_fwd(w2, _dev(xs), y, ws)
+    got, clean = y.cpu().numpy(), clean.cpu().numpy()
+    touched = np.zeros((m, n), dtype=bool)
+    for jj, cc in ((7, 3), (k - 1, n - 1), (70, 0), (71, 1)):
+        touched[a[:, jj] != 0, cc] = True
+    touched[r] = True
+    np.testing.assert_allclose(got[~touched], clean[~touched], rtol=1e-4, atol=1e-6 * float(np.abs(clean).max()))
+    with np.errstate(all="ignore"):
+        for i, c in np.argwhere(touched)[:: max(1, touched.sum() // 2000)]:
+            js = np.flatnonzero(a2[i])
+            want = np.float32(0)
+            for t in js:
+                want = np.float32(np.float64(a2[i, t]) * np.float64(xs[t, c]) + np.float64(want))
+            if np.isfinite(want):
+                S = np.abs(a2[i, js].astype(np.float64) * xs[js, c]).sum()
+                assert abs(got[i, c] - want) <= 1e-6 * S, (i, c, got[i, c], want)
+            else:
+                assert np.array_equal(got[i, c], want, equal_nan=True), (i, c, got[i, c], want)
+    assert ws.status()[0] == 0
+
+
 # --- weight gradients ----------------------------------------------------------
 
 @pytest.mark.parametrize("m,k,n", [(300, 784, 64), (10, 500, 128), (20, 25, 9000), (129, 67, 33),
