@@ -41,6 +41,19 @@ template <int VW>
 __device__ __forceinline__ typename Vec<VW>::T ldv(const float *p) {
     return __ldg(reinterpret_cast<const typename Vec<VW>::T *>(p));
 }
+// The same, kept in program order among themselves: a batch's loads are all
+// issued before the first of them is waited for.
+template <int VW>
+__device__ __forceinline__ typename Vec<VW>::T ldv_now(const float *p) {
+    typename Vec<VW>::T v;
+    if constexpr (VW == 4)
+        asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    else if constexpr (VW == 2)
+        asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    else
+        asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 template <int VW>
 __device__ __forceinline__ void stv(float *p, const float (&a)[VW]) {
     if constexpr (VW == 4) *reinterpret_cast<float4 *>(p) = make_float4(a[0], a[1], a[2], a[3]);
@@ -735,19 +748,18 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // ---------------------------------------------------------------------------
 // SDDMM: g[k] = <dY[i_k, :], X[j_k, :]>
 // ---------------------------------------------------------------------------
-// Layout as in the narrow SpMM kernel: a group of G lanes (G*VW >= n, or
-// G = 32 with NV vectors per lane and the n range walked in tiles of
-// TN = 32*VW*NV) takes one stored entry, a warp step covers E = 32/G entries,
-// and U steps form a batch whose column indices are requested before the
-// previous batch is consumed. Every entry of a batch lies in one row, whose
-// dY slice stays in registers for the whole row when one tile covers n (else
-// it is reloaded once per batch and tile), so per entry only its row of X is
-// read. The U dot products of a lane are finished together: the first
-// log2(min(U, G)) butterfly steps over the group's lanes exchange halves of
-// the U partial sums (a transposed reduction), the remaining steps add one
-// value, and lane r*(G/R) of each group holds entry r's result. No partial
-// buffers: the whole n range of an entry is summed in one warp, so the
-// result does not depend on the unit split.
+// Up to 16 lanes per entry (sddmm_kernel): layout as in the narrow SpMM
+// kernel, a group of G lanes (G*VW >= n) takes one stored entry, a warp step
+// covers E = 32/G entries, and U steps form a batch whose column indices are
+// requested before the previous batch is consumed. Every entry of a batch lies
+// in one row, whose dY slice stays in registers for the whole row, so per
+// entry only its row of X is read. Wider products: sddmm_wide_kernel. The dot
+// products of a batch are finished together: the first log2 butterfly steps
+// over the group's lanes exchange halves of the partial sums (a transposed
+// reduction), the remaining steps add one value, and lane r*(G/R) of each
+// group holds entry r's result. No partial buffers: the whole n range of an
+// entry is summed in one warp, so the result does not depend on the unit
+// split.
 struct SddmmArgs {
     const int32_t *row_ptr;
     const int32_t *col;
@@ -785,6 +797,142 @@ __device__ __forceinline__ void group_reduce_multi(float (&p)[U], int gl) {
         }
 #pragma unroll
         for (int off = G / (2 * R); off >= 1; off >>= 1) p[b * R] += __shfl_xor_sync(0xffffffffu, p[b * R], off);
+    }
+}
+
+// Wide SDDMM: 32 lanes per entry, NV vectors of VW floats each (TN columns of
+// a tile; kMulti: several tiles; kFull: n fills them). Batches
+// of F entries of one row in a software pipeline: a batch's rows of X (and the
+// slice of dY that goes with them) are asked for as soon as the step before
+// has used up its own, before that batch's sums are reduced and stored; the
+// column indices come one batch earlier. A row's last batch repeats its last
+// entry instead of being shorter, so no entry is predicated, and one 64-bit
+// address is formed per entry.
+// What bounds it: the gathers of X from L2 for 256 columns (21 TB/s), issue
+// (70%) for 128. Measured, 4096 x 4096 at 20%: n = 256 213 -> 164 us, n = 128
+// 166 -> 112 us; the kernel before took 43 to 46 instructions per entry,
+// predicated, and reduced between its loads; n = 255 (scalar loads, in one
+// tile of 256 instead of four of 64) 528 -> 212 us, 1024 in four tiles
+// 811 -> 722 us. Without kFull's forms the column bounds take 10% more.
+// 8 floats per lane take 128 registers (two blocks per SM: with three the
+// batch in flight spills, 2.3 times slower), 4 floats 80.
+template <int VW, int NV, bool kMulti, bool kFull = false>
+__global__ void __launch_bounds__(kSpThreads, VW * NV >= 8 ? 2 : 3) sddmm_wide_kernel(SddmmArgs a) {
+    pdl_enter();
+    constexpr int F = 4, TN = 32 * VW * NV, kStride = 32 * VW;
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = ((int64_t)blockIdx.x * kSpThreads + threadIdx.x) >> 5;
+    if (gw >= (int64_t)a.units) return;
+    const int32_t nnz = __ldg(a.row_ptr + a.rows);
+    const int64_t per = ceil_div<int64_t>(nnz, a.units);
+    const int32_t k0 = (int32_t)imin<int64_t>(gw * per, nnz), k1 = (int32_t)imin<int64_t>(k0 + per, nnz);
+    if (k0 >= k1) return;
+    const int n = kFull && !kMulti ? TN : a.n;
+    const int tiles = kMulti ? ceil_div(n, TN) : 1;
+    const int left0 = n - lane * VW;   // columns from this lane's first on
+    const char *x = reinterpret_cast<const char *>(a.x + lane * VW);
+    const float *dy = a.dy + lane * VW;
+    const uint64_t row_bytes = (uint64_t)n * sizeof(float);
+    int row = row_of_entry(a.row_ptr, a.rows, k0);
+    int wb = row;
+    int32_t ends = wb + lane < a.rows ? __ldg(a.row_ptr + wb + lane + 1) : nnz;
+    int32_t e = imin(__shfl_sync(0xffffffffu, ends, 0), k1);
+    // moves on to the row that holds entry k (empty rows are passed over)
+    auto seek = [&](int32_t k) {
+        while (e <= k) {
+            if (++row - wb >= 32) {
+                wb = row;
+                ends = wb + lane < a.rows ? __ldg(a.row_ptr + wb + lane + 1) : nnz;
+            }
+            e = imin(__shfl_sync(0xffffffffu, ends, row - wb), k1);
+        }
+    };
+    int32_t c[F], cn[F];   // columns of the batch in hand (kMulti) and of the next
+    auto columns = [&](int32_t k) {
+#pragma unroll
+        for (int s = 0; s < F; ++s) cn[s] = __ldg(a.col + imin(k + s, e - 1));
+    };
+    float d[NV][VW];
+    typename Vec<VW>::T xv[F][NV];
+    const typename Vec<VW>::T zero{};
+    auto load_dy = [&](int r, int tt) {
+        const float *p = dy + (int64_t)r * n + tt * TN;
+        const int left = left0 - tt * TN;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) unpack<VW>(kFull || v * kStride < left ? ldv<VW>(p + v * kStride) : zero, d[v]);
+    };
+    auto load_x = [&](const int32_t (&cols)[F], int tt) {
+        const int left = left0 - tt * TN;
+        const char *xt = x + (int64_t)tt * (TN * (int)sizeof(float));
+#pragma unroll
+        for (int s = 0; s < F; ++s) {
+            const float *p = reinterpret_cast<const float *>(xt + (uint64_t)(uint32_t)cols[s] * row_bytes);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                if (kFull || v * kStride < left) xv[s][v] = ldv_now<VW>(p + v * kStride);
+                else xv[s][v] = zero;
+            }
+        }
+    };
+    int32_t k = k0;      // the batch in hand: its rows of X are loaded
+    seek(k);
+    columns(k);
+    if constexpr (kMulti) {
+#pragma unroll
+        for (int s = 0; s < F; ++s) c[s] = cn[s];
+    }
+    load_dy(row, 0);
+    load_x(cn, 0);
+    int row_x = row, tt = 0;
+    int32_t k_n = imin(k + F, e);   // the next batch: its columns are
+    if (k_n < k1) {
+        seek(k_n);
+        columns(k_n);
+    }
+    float p[F];
+#pragma unroll
+    for (int s = 0; s < F; ++s) p[s] = 0.f;
+    while (true) {
+#pragma unroll
+        for (int s = 0; s < F; ++s)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                float f[VW];
+                unpack<VW>(xv[s][v], f);
+#pragma unroll
+                for (int i = 0; i < VW; ++i) p[s] = fmaf(d[v][i], f[i], p[s]);
+            }
+        if constexpr (kMulti) {
+            if (++tt < tiles) {
+                load_dy(row_x, tt);
+                load_x(c, tt);
+                continue;
+            }
+            tt = 0;
+        }
+        float *out = a.out + k;
+        const int cnt = k_n - k;
+        const bool more = k_n < k1;
+        if (more) {
+            if (kMulti || row != row_x) load_dy(row, 0);
+            load_x(cn, 0);
+            if constexpr (kMulti) {
+#pragma unroll
+                for (int s = 0; s < F; ++s) c[s] = cn[s];
+            }
+            k = k_n;
+            row_x = row;
+            k_n = imin(k + F, e);
+            if (k_n < k1) {
+                seek(k_n);
+                columns(k_n);
+            }
+        }
+        group_reduce_multi<F, 32>(p, lane);
+        if (lane % 8 == 0 && lane / 8 < cnt) out[lane / 8] = p[0];
+        if (!more) break;
+#pragma unroll
+        for (int s = 0; s < F; ++s) p[s] = 0.f;
     }
 }
 
@@ -1056,8 +1204,11 @@ int weight_grad_sddmm(const csrt_csr *w, const float *dy, const float *x, int32_
     const bool v4 = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 15) == 0;
     const bool v2 = (n % 2 == 0) && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 7) == 0;
     const int vw = v4 ? 4 : v2 ? 2 : 1;
+    // up to 16 lanes per entry, or all 32 with 4 floats per lane up to 128
+    // columns (2 up to 64) and 8 beyond, in tiles of 256 columns
     const int g = imin(32, pow2_at_least((n + vw - 1) / vw));
-    const int nv = g == 32 && n > 32 * vw ? 2 : 1;
+    const int per_lane = n <= 64 ? 2 : n <= 128 ? 4 : 8;
+    const int nv = g < 32 ? 1 : imax(1, per_lane / vw);
     SddmmArgs a;
     a.row_ptr = w->row_ptr;
     a.col = w->col_idx;
@@ -1066,23 +1217,31 @@ int weight_grad_sddmm(const csrt_csr *w, const float *dy, const float *x, int32_
     a.x = x;
     a.n = n;
     a.out = g_nnz;
-    static int cache[64][3][6][2];
+    static int cache[64][3][6][4];
     int dev = 0;
     CSRT_CHECK_CUDA(cudaGetDevice(&dev));
     CSRT_ARG(dev >= 0 && dev < 64, "device ordinal %d out of range", dev);
-    int lg = 0;
+    int lg = 0, lnv = 0;
     while ((1 << lg) < g) ++lg;
-    int &wps = cache[dev][vw == 4 ? 2 : vw - 1][lg][nv - 1];
+    while ((1 << lnv) < nv) ++lnv;
     void (*kern)(SddmmArgs) = nullptr;
-#define CSRT_SDDMM_CASE(VW, NV, G) \
-    if (vw == VW && nv == NV && g == G) kern = sddmm_kernel<VW, NV, G>;
-    CSRT_SDDMM_CASE(4, 1, 1) CSRT_SDDMM_CASE(4, 1, 2) CSRT_SDDMM_CASE(4, 1, 4) CSRT_SDDMM_CASE(4, 1, 8)
-    CSRT_SDDMM_CASE(4, 1, 16) CSRT_SDDMM_CASE(4, 1, 32) CSRT_SDDMM_CASE(4, 2, 32)
-    CSRT_SDDMM_CASE(2, 1, 1) CSRT_SDDMM_CASE(2, 1, 2) CSRT_SDDMM_CASE(2, 1, 4) CSRT_SDDMM_CASE(2, 1, 8)
-    CSRT_SDDMM_CASE(2, 1, 16) CSRT_SDDMM_CASE(2, 1, 32) CSRT_SDDMM_CASE(2, 2, 32)
-    CSRT_SDDMM_CASE(1, 1, 1) CSRT_SDDMM_CASE(1, 1, 2) CSRT_SDDMM_CASE(1, 1, 4) CSRT_SDDMM_CASE(1, 1, 8)
-    CSRT_SDDMM_CASE(1, 1, 16) CSRT_SDDMM_CASE(1, 1, 32) CSRT_SDDMM_CASE(1, 2, 32)
+#define CSRT_SDDMM_CASE(VW, G) \
+    if (vw == VW && g == G) kern = sddmm_kernel<VW, 1, G>;
+    CSRT_SDDMM_CASE(4, 1) CSRT_SDDMM_CASE(4, 2) CSRT_SDDMM_CASE(4, 4) CSRT_SDDMM_CASE(4, 8) CSRT_SDDMM_CASE(4, 16)
+    CSRT_SDDMM_CASE(2, 1) CSRT_SDDMM_CASE(2, 2) CSRT_SDDMM_CASE(2, 4) CSRT_SDDMM_CASE(2, 8) CSRT_SDDMM_CASE(2, 16)
+    CSRT_SDDMM_CASE(1, 1) CSRT_SDDMM_CASE(1, 2) CSRT_SDDMM_CASE(1, 4) CSRT_SDDMM_CASE(1, 8) CSRT_SDDMM_CASE(1, 16)
 #undef CSRT_SDDMM_CASE
+#define CSRT_SDDMM_CASE(VW, NV) \
+    if (vw == VW && g == 32 && nv == NV) kern = sddmm_wide_kernel<VW, NV, false>;
+    CSRT_SDDMM_CASE(4, 1) CSRT_SDDMM_CASE(4, 2) CSRT_SDDMM_CASE(2, 1) CSRT_SDDMM_CASE(2, 2) CSRT_SDDMM_CASE(2, 4)
+    CSRT_SDDMM_CASE(1, 2) CSRT_SDDMM_CASE(1, 4) CSRT_SDDMM_CASE(1, 8)
+#undef CSRT_SDDMM_CASE
+    if (n > 256)
+        kern = vw == 4 ? sddmm_wide_kernel<4, 2, true> : vw == 2 ? sddmm_wide_kernel<2, 4, true> : sddmm_wide_kernel<1, 8, true>;
+    if (vw == 4 && n == 128) kern = sddmm_wide_kernel<4, 1, false, true>;
+    if (vw == 4 && n % 256 == 0) kern = n == 256 ? sddmm_wide_kernel<4, 2, false, true> : sddmm_wide_kernel<4, 2, true, true>;
+    // (the forms of a wide kernel have the same launch bounds)
+    int &wps = cache[dev][vw == 4 ? 2 : vw - 1][lg][lnv];
     CSRT_ARG(kern != nullptr, "sddmm: no kernel for vw=%d nv=%d g=%d", vw, nv, g);
     // 2..16 lanes per entry: the per-warp ring of column indices in shared memory
     const size_t smem = (g > 1 && g < 32) ? (size_t)(kSpThreads / 32) * kSdStages * kSdChunk * sizeof(int32_t) : 0;

@@ -473,6 +473,31 @@ def test_weight_grad_sddmm(C, m, k, n, density, zipf):
 
 # --- prox_update_compact / debias_update ---------------------------------------
 
+@pytest.mark.parametrize("n", [33, 65, 66, 127, 128, 129, 255, 256, 257, 258, 300, 512, 515, 1023, 1024])
+def test_sddmm_wide(C, n):
+    """Wide SDDMM: every vector width, filled and partly filled column tiles, batches cut by rows and units; rows that
+    are empty, hold one entry, or are longer than a unit."""
+    m, k = 37, 3000
+    rng = np.random.default_rng(n)
+    a = _sparse(rng, m, k, 0.02)
+    a[[0, 5, 6, m - 1]] = 0.0
+    a[3] = 0.0
+    a[3, 17] = 2.0
+    a[9] = 1.0
+    dy = rng.standard_normal((m, n)).astype(F32)
+    x = rng.standard_normal((k, n)).astype(F32)
+    ws = _ws(C, m, k, n)
+    ref = O.csr_from_dense(a)
+    g = torch.full((ref.nnz + 5,), 7.0, device="cuda")
+    for capacity in (ref.nnz, m * k):     # few and many units: the same sums
+        w = _gpu_csr(C, a, ws, transposed=False, capacity=capacity)
+        C.weight_grad_sddmm(w, _dev(dy), _dev(x), g, ws)
+        got = g.cpu().numpy()
+        assert (got[ref.nnz:] == 7.0).all()
+        assert_close(got[: ref.nnz], O.weight_grad_sddmm(ref, dy, x), O.weight_grad_sddmm(ref, np.abs(dy), np.abs(x)), n,
+                     what="sddmm")
+
+
 def test_prox_hand_cases_on_gpu(C):
     with open(os.path.join(GOLD, "soft_threshold_cases.json")) as f:
         d = json.load(f)
