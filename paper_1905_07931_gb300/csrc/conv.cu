@@ -7,79 +7,117 @@
 // window, so this kernel reads the input in place: the unfolded matrix, which
 // is k*k times larger than the input, is never written or read.
 //
-// One block per (output channel m, tile of output pixels). The block stages
-// the channel's stored taps in shared memory as (weight, input offset) pairs;
-// tap k = (c*k + ky)*k + kx of the CSR row reads input pixel
-// x[c][b][oy+ky][ox+kx], at offset c*B*H*W + ky*W + kx from the window's
-// corner x[0][b][oy][ox]. Each thread accumulates kConvPer output pixels
-// (consecutive pixels go to consecutive threads, so the input reads of a warp
-// are contiguous along ox) over the taps in CSR order with one fused
-// multiply-add per tap, then applies the bias and ReLU. The input window
-// of a block is reused by every tap from L1.
+// One block per (tile of output pixels, group of output channels). A block
+// stages the taps of its channels in shared memory as (input offset, weight)
+// pairs: tap t = (c*k + ky)*k + kx of a CSR row reads input pixel
+// x[c][b][oy+ky][ox+kx], c*B*H*W + ky*W + kx elements from the window's
+// corner x[0][b][oy][ox]. Each thread accumulates its output pixels over the
+// taps of one channel after the other in CSR order, with one fused
+// multiply-add per tap, then applies the bias and ReLU. A window is reused by
+// all taps of all channels of the block from L1.
+//
+// What bounds it: the L1 reads, one per tap and pixel, once the index work is
+// out of the way. Dividing a pixel number into sample, row and column in 64
+// bits for every channel took more time than the taps of a layer with few of
+// them, so the channels of a group share the corners, and inputs under 4 GiB
+// (every one of practical size) use 32-bit offsets: one add, one load and one
+// multiply-add per tap and pixel. LeNet-5 at 1000 images: conv1 (20 channels,
+// 7.9 taps each) 61.1 -> 29.4 us; conv2 (50 channels, 42 taps) 51.5 -> 41.3 us,
+// and 36.1 us with the lane order below.
+//
+// Lane order: a warp that reads 32 / Wo consecutive output rows for one tap
+// touches rows W words apart, which share banks unless W is a multiple of Wo.
+// Where Wo divides 32, the warp takes rows 2^e apart instead, with the
+// smallest e <= 3 that makes (W << e) an odd multiple of Wo modulo 32: its
+// reads then fall into 32 different banks (W = 12, Wo = 8, rows 0 2 4 6: conv2
+// 41.3 -> 36.1 us; 32 x 32 channels of 20 x 20, Wo = 16: 86.7 -> 69.9 us). The
+// warps of a block take the rows between, so the pixels of a block and the sum
+// of each pixel are the same as without.
 #include "common.cuh"
 
 namespace csrt {
 
 constexpr int kConvThreads = 256;
-constexpr int kConvPer = 4;          // output pixels per thread
+constexpr int kConvPer = 4;          // output pixels per thread, large outputs
 constexpr int kConvTaps = 1024;      // taps staged per round
+constexpr int kConvGroup = 32;       // most output channels per block
+constexpr int kConvBlocksPerSM = 16;  // blocks per SM to keep when channels share a block
 
+template <typename I>
+struct ConvTap {
+    I off;     // bytes from a window's corner to the tap's input
+    float w;
+};
+
+// I: uint32_t when the input's bytes and the pixel count fit, else uint64_t.
+template <typename I, int kPer>
 __global__ void __launch_bounds__(kConvThreads) conv_sparse_fwd_kernel(
-    const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, const float *__restrict__ val,
-    const float *__restrict__ x, int32_t cin, int32_t b, int32_t h, int32_t w, int32_t k,
+    const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, const float *__restrict__ val, int32_t rows,
+    int32_t group, int32_t ox_bits, int32_t step_bits, const float *__restrict__ x, int32_t b, int32_t h, int32_t w, int32_t k,
     const float *__restrict__ bias, int32_t relu, float *__restrict__ y) {
     pdl_enter();
-    __shared__ float s_w[kConvTaps];
-    __shared__ int64_t s_off[kConvTaps];
-    const int ho = h - k + 1, wo = w - k + 1;
-    const int64_t plane = (int64_t)b * h * w;             // one input channel
-    const int64_t npix = (int64_t)b * ho * wo;            // output pixels per channel
-    const int m = blockIdx.y;
-    const int64_t p0 = (int64_t)blockIdx.x * kConvThreads * kConvPer + threadIdx.x;
-    // window corner of each of this thread's pixels
-    int64_t corner[kConvPer];
-    bool valid[kConvPer];
+    __shared__ ConvTap<I> s_tap[kConvTaps];
+    __shared__ int32_t s_end[kConvGroup];
+    const I ho = h - k + 1, wo = w - k + 1;
+    const I plane = (I)b * h * w;              // one input channel
+    const I npix = (I)b * ho * wo;             // output pixels per channel
+    const int m0 = blockIdx.y * group, m1 = imin(m0 + group, rows);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int step_mask = (1 << step_bits) - 1, ox_mask = (1 << ox_bits) - 1;
+    // the thread's place in its block's pixels: the lane order described above
+    const int t = (lane & ox_mask) | (warp & step_mask) << ox_bits | (lane >> ox_bits) << (ox_bits + step_bits) |
+                  (warp >> step_bits) << (5 + step_bits);
+    const I p0 = (I)blockIdx.x * (kConvThreads * kPer) + t;
+    I corner[kPer];   // bytes to the window corner of each pixel; past the last pixel, of pixel 0
 #pragma unroll
-    for (int q = 0; q < kConvPer; ++q) {
-        const int64_t p = p0 + (int64_t)q * kConvThreads;
-        valid[q] = p < npix;
-        const int64_t pp = valid[q] ? p : 0;
-        const int64_t s = pp / ((int64_t)ho * wo);
-        const int rem = (int)(pp - s * ho * wo);
-        const int oy = rem / wo, ox = rem - oy * wo;
-        corner[q] = (s * h + oy) * w + ox;
+    for (int q = 0; q < kPer; ++q) {
+        const I p = p0 + q * kConvThreads;
+        const I pp = p < npix ? p : 0;
+        const I s = pp / (ho * wo);
+        const I rem = pp - s * (ho * wo);
+        const I oy = rem / wo, ox = rem - oy * wo;
+        corner[q] = ((s * h + oy) * w + ox) * 4;
     }
-    float acc[kConvPer];
+    const int32_t t0 = __ldg(row_ptr + m0), t1 = __ldg(row_ptr + m1);
+    if ((int)threadIdx.x < m1 - m0) s_end[threadIdx.x] = __ldg(row_ptr + m0 + threadIdx.x + 1);
+    float acc[kPer];
 #pragma unroll
-    for (int q = 0; q < kConvPer; ++q) acc[q] = 0.f;
-    const int32_t t0 = __ldg(row_ptr + m), t1 = __ldg(row_ptr + m + 1);
-    for (int32_t tb = t0; tb < t1; tb += kConvTaps) {
+    for (int q = 0; q < kPer; ++q) acc[q] = 0.f;
+    int m = m0;
+    for (int32_t tb = t0;; tb += kConvTaps) {
         const int nt = imin(kConvTaps, t1 - tb);
+        const bool last = t1 - tb <= kConvTaps;
         __syncthreads();   // the previous round's taps are consumed
         for (int i = threadIdx.x; i < nt; i += kConvThreads) {
             const int tap = __ldg(col + tb + i);
             const int c = tap / (k * k), kk = tap - c * k * k;
             const int ky = kk / k, kx = kk - ky * k;
-            s_off[i] = (int64_t)c * plane + (int64_t)ky * w + kx;
-            s_w[i] = __ldg(val + tb + i);
+            s_tap[i] = {((I)c * plane + (I)ky * w + kx) * 4, __ldg(val + tb + i)};
         }
         __syncthreads();
-        for (int i = 0; i < nt; ++i) {
-            const float wt = s_w[i];
-            const int64_t off = s_off[i];
+        for (int i = 0; m < m1; ++m) {
+            const int end = s_end[m - m0] - tb;
+            const int stop = imin(end, nt);
+#pragma unroll 4
+            for (; i < stop; ++i) {
+                const ConvTap<I> tap = s_tap[i];
 #pragma unroll
-            for (int q = 0; q < kConvPer; ++q)
-                if (valid[q]) acc[q] = fmaf(wt, __ldg(x + corner[q] + off), acc[q]);
+                for (int q = 0; q < kPer; ++q)
+                    acc[q] = fmaf(tap.w, __ldg((const float *)((const char *)x + (I)(corner[q] + tap.off))), acc[q]);
+            }
+            if (end > nt && !last) break;   // the channel's taps go on in the next round
+            const float bm = bias ? __ldg(bias + m) : 0.f;
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                float v = acc[q];
+                acc[q] = 0.f;
+                if (bias) v = __fadd_rn(v, bm);
+                if (relu) v = fmaxf(v, 0.f);
+                const I p = p0 + q * kConvThreads;
+                if (p < npix) y[(int64_t)m * (int64_t)npix + (int64_t)p] = v;
+            }
         }
-    }
-    const float bm = bias ? __ldg(bias + m) : 0.f;
-#pragma unroll
-    for (int q = 0; q < kConvPer; ++q) {
-        if (!valid[q]) continue;
-        float v = acc[q];
-        if (bias) v = __fadd_rn(v, bm);
-        if (relu) v = fmaxf(v, 0.f);
-        y[(int64_t)m * npix + p0 + (int64_t)q * kConvThreads] = v;
+        if (last) break;
     }
 }
 
@@ -98,10 +136,36 @@ extern "C" int csrt_conv2d_sparse_fwd(const csrt_csr *w, const float *x, int32_t
     if (npix == 0) return CSRT_OK;
     CSRT_ARG(x != nullptr && y != nullptr, "x or y is NULL");
     CSRT_ARG(w->capacity == 0 || (w->col_idx && w->val), "col_idx/val NULL");
-    const int64_t blocks = ceil_div<int64_t>(npix, (int64_t)kConvThreads * kConvPer);
-    CSRT_ARG(blocks < ((int64_t)1 << 31), "too many output pixels");
-    launch_pdl(conv_sparse_fwd_kernel, dim3((unsigned)blocks, (unsigned)w->rows), dim3(kConvThreads), 0,
-               as_stream(stream), w->row_ptr, w->col_idx, w->val, x, c, b, h, wd, k, bias, relu, y);
+    const int64_t tiles4 = ceil_div<int64_t>(npix, (int64_t)kConvThreads * kConvPer);
+    CSRT_ARG(tiles4 < ((int64_t)1 << 31), "too many output pixels");
+    // byte offsets in 32 bits; the pixel numbers of the last tile run past npix by less than a tile
+    const bool narrow = (int64_t)c * b * h * wd < ((int64_t)1 << 30) && npix < ((int64_t)1 << 31);
+    // Four pixels per thread share the staged taps and keep four loads in
+    // flight; with fewer than two blocks per SM, one pixel per thread spreads
+    // the work over more threads instead (conv2 of LeNet-5 at 64 images, 200
+    // blocks: 7.8 us with four, 6.2 us with one; conv1 at 64, 720 blocks: 4.9 us
+    // with four, 7.3 us with one).
+    const bool small = narrow && tiles4 * w->rows < (int64_t)num_sms() * 2;
+    const int64_t tiles = small ? ceil_div<int64_t>(npix, kConvThreads) : tiles4;
+    // As many channels per block as leave kConvBlocksPerSM blocks per SM
+    // (conv1 / conv2 of LeNet-5 at 1000 images with 8, 16 and 32 per SM: 26.9 /
+    // 46.6, 27.5 / 40.8, 30.6 / 40.7 us).
+    const int group = (int)imax<int64_t>(
+        1, imin<int64_t>(kConvGroup, tiles * w->rows / ((int64_t)num_sms() * kConvBlocksPerSM)));
+    int ox_bits = 5, step_bits = 0;   // consecutive pixels in consecutive lanes
+    const int wo = wd - k + 1;
+    if (wo < 32 && 32 % wo == 0)
+        for (int e = 0; e <= 3; ++e)
+            if (((int64_t)wd << e) % (2 * wo) == wo) {
+                while ((1 << ox_bits) > wo) --ox_bits;
+                step_bits = e;
+                break;
+            }
+    const auto kern = small ? conv_sparse_fwd_kernel<uint32_t, 1>
+                      : narrow ? conv_sparse_fwd_kernel<uint32_t, kConvPer> : conv_sparse_fwd_kernel<uint64_t, kConvPer>;
+    launch_pdl(kern, dim3((unsigned)tiles, (unsigned)ceil_div(w->rows, group)), dim3(kConvThreads), 0,
+               as_stream(stream), w->row_ptr, w->col_idx, w->val, w->rows, group, ox_bits, step_bits, x, b, h, wd, k,
+               bias, relu, y);
     count_launch();
     return check_launch("conv_sparse_fwd_kernel");
 }

@@ -1061,6 +1061,48 @@ def test_conv2d_sparse_fwd_against_oracle(C, cout, cin, b, h, w, k, density, rel
     assert_close(y.cpu().numpy(), ref, bound, (np.diff(ref_w.row_ptr) + 1)[:, None], what="conv2d_sparse_fwd")
 
 
+@pytest.mark.parametrize("cout,cin,b,h,w,k,density,relu", [
+    (40, 1, 217, 28, 28, 5, 0.3, False),    # channels share a block, the last group is short
+    (64, 8, 901, 20, 20, 5, 1.0, True),     # a group's taps need more than one round, rows 4 apart
+    (37, 20, 64, 12, 12, 5, 0.08, False),   # one pixel per thread, rows 2 apart
+    (64, 3, 300, 18, 18, 3, 0.4, False),    # rows 8 apart
+    (33, 2, 150, 9, 32, 1, 0.5, True),      # one output row per warp
+    (48, 4, 333, 11, 7, 4, 0.3, False),     # four columns per output row
+])
+def test_conv2d_sparse_fwd_blocks(C, cout, cin, b, h, w, k, density, relu):
+    """Shared blocks, rounds and lane orders against the unfolded product in 64 bits."""
+    rng = np.random.default_rng(cout + cin + b)
+    wt = _sparse(rng, cout, cin * k * k, density)
+    x = _dev(rng.standard_normal((cin, b, h, w)).astype(F32))
+    bias = _dev(rng.standard_normal(cout).astype(F32))
+    W = _gpu_csr(C, wt, _ws(C, cout, cin * k * k, 1), transposed=False)
+    y = torch.full((cout, b * (h - k + 1) * (w - k + 1)), float("nan"), device="cuda")
+    C.conv2d_sparse_fwd(W, x.reshape(cin, -1), cin, b, h, w, k, bias, relu, y)
+    wd = _dev(wt).double()
+    cols = x.double().unfold(2, k, 1).unfold(3, k, 1).permute(0, 4, 5, 1, 2, 3).reshape(cin * k * k, -1)
+    ref = wd @ cols + bias.double()[:, None]
+    bound = wd.abs() @ cols.abs() + bias.double().abs()[:, None]
+    terms = (wd != 0).sum(1, keepdim=True) + 1
+    if relu:
+        ref = ref.clamp_min(0.0)
+    # one rounding per tap and one for the bias, each within 2^-24 of a partial sum
+    assert bool(((y.double() - ref).abs() <= 1.01 * 2.0 ** -24 * terms * bound + 1e-37).all())
+
+
+def test_conv2d_sparse_fwd_wide_offsets(C):
+    """An input of more than 4 GiB: offsets in 64 bits, exact for one tap of a 1 x 1 filter."""
+    h = w = 32
+    b = (1 << 20) + 3
+    W = _gpu_csr(C, np.array([[0.75], [0.0]], F32), _ws(C, 2, 1, 1), transposed=False)
+    x = torch.randn(1, b * h * w, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    bias = _dev(np.array([0.3, -1.5], F32))
+    y = torch.empty(2, b * h * w, device="cuda")
+    C.conv2d_sparse_fwd(W, x, 1, b, h, w, 1, bias, False, y)
+    assert bool((y[1] == -1.5).all())
+    x.mul_(0.75).add_(bias[0])
+    assert torch.equal(y[0], x[0])
+
+
 # --- failure detection: bounded waits give up and report ---------------------
 
 def test_bounded_waits_give_up_and_report(C):
