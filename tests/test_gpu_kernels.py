@@ -1103,6 +1103,26 @@ def test_conv2d_sparse_fwd_wide_offsets(C):
     assert torch.equal(y[0], x[0])
 
 
+@pytest.mark.parametrize("off", [0, 1])
+def test_maxpool2_fwd_alignment(C, off):
+    """Pairs read in one load where x is 8-byte aligned, one by one where not; ties take the first, NaN never wins."""
+    c, b, h, w = 3, 7, 10, 6
+    rng = np.random.default_rng(off)
+    x = rng.integers(-2, 3, (c, b, h, w)).astype(F32)
+    x[0, 0, 0, 1] = np.nan
+    xd = torch.empty(x.size + 1, device="cuda")[off:off + x.size]
+    xd.copy_(torch.from_numpy(x.reshape(-1)))
+    y = torch.empty(c * b * (h // 2) * (w // 2), device="cuda")
+    idx = torch.full((y.numel(),), -1, dtype=torch.int8, device="cuda")
+    C.maxpool2_fwd(xd, c, b, h, w, y, idx)
+    win = x.reshape(c, b, h // 2, 2, w // 2, 2).transpose(0, 1, 2, 4, 3, 5).reshape(-1, 4)
+    best = np.zeros(len(win), np.int8)
+    for q in range(1, 4):
+        best[win[:, q] > win[np.arange(len(win)), best]] = q
+    assert np.array_equal(idx.cpu().numpy(), best)
+    assert np.array_equal(y.cpu().numpy(), win[np.arange(len(win)), best])
+
+
 # --- failure detection: bounded waits give up and report ---------------------
 
 def test_bounded_waits_give_up_and_report(C):
