@@ -274,6 +274,48 @@ __global__ void flatten_kernel(const float *__restrict__ in, int32_t c, int32_t 
     }
 }
 
+// Both directions are one transposition per channel, out[ci][j][i] =
+// in[ci][i][j]: a 32 x 32 tile through shared memory makes the reads and the
+// writes contiguous. One element per thread with a stride between lanes asks
+// L2 for a sector per element and divides twice in 64 bits: 50 x 1000 x 16
+// 5.4 -> 3.1 us, 20 x 1000 x 576 50.4 -> 15.1 us and back 68.6 -> 15.7 us.
+constexpr int kFlatTile = 32;
+constexpr int kFlatMin = 12;
+
+__global__ void __launch_bounds__(256) flatten_tile_kernel(const float *__restrict__ in, int32_t rows, int32_t cols,
+                                                           float *__restrict__ out) {
+    pdl_enter();
+    __shared__ float s_tile[kFlatTile][kFlatTile + 1];
+    const int64_t base = (int64_t)blockIdx.z * rows * cols;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * kFlatTile, j0 = blockIdx.y * kFlatTile;
+#pragma unroll
+    for (int r = 0; r < kFlatTile; r += 8) {
+        const int i = i0 + r + ty, j = j0 + tx;
+        if (i < rows && j < cols) s_tile[r + ty][tx] = __ldg(in + base + (int64_t)i * cols + j);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kFlatTile; r += 8) {
+        const int j = j0 + r + ty, i = i0 + tx;
+        if (i < rows && j < cols) out[base + (int64_t)j * rows + i] = s_tile[tx][r + ty];
+    }
+}
+
+static void launch_flatten(const float *in, int32_t c, int32_t b, int32_t hw, float *out, int inverse, void *stream) {
+    const int64_t total = (int64_t)c * b * hw;
+    const int32_t rows = inverse ? hw : b, cols = inverse ? b : hw;
+    // Narrow matrices leave most of a tile idle (1000 x 4 x 784: 11.9 us one by
+    // one, 26.7 us by tiles; 500 x 6 x 1600: 16.1, 26.9; 100 x 2000 x 12: 9.4,
+    // 6.9); the other two are the limits of the grid.
+    if (imin(b, hw) >= kFlatMin && c <= 65535 && ceil_div(cols, kFlatTile) <= 65535) {
+        launch_pdl(flatten_tile_kernel, dim3(ceil_div(rows, kFlatTile), ceil_div(cols, kFlatTile), c), dim3(256), 0,
+                   as_stream(stream), in, rows, cols, out);
+    } else {
+        launch_pdl(flatten_kernel, dim3(grid_for(total)), dim3(256), 0, as_stream(stream), in, c, b, hw, out, inverse);
+    }
+}
+
 // FP32 FMA throughput probe (the roof of the CUDA-core products): every
 // thread runs kFmaChains independent fused multiply-add chains
 // (x <- x*b + c with |b| < 1, so the values stay finite) for `iters` rounds
@@ -404,7 +446,7 @@ int csrt_flatten(const float *x, int32_t c, int32_t b, int32_t hw, float *xf, vo
     const int64_t total = (int64_t)c * b * hw;
     if (total == 0) return CSRT_OK;
     CSRT_ARG(x && xf, "NULL pointer");
-    launch_pdl(flatten_kernel, dim3(grid_for(total)), dim3(256), 0, as_stream(stream), x, c, b, hw, xf, 0);
+    launch_flatten(x, c, b, hw, xf, 0, stream);
     count_launch();
     return check_launch("flatten_kernel");
 }
@@ -414,7 +456,7 @@ int csrt_unflatten(const float *xf, int32_t c, int32_t b, int32_t hw, float *x, 
     const int64_t total = (int64_t)c * b * hw;
     if (total == 0) return CSRT_OK;
     CSRT_ARG(x && xf, "NULL pointer");
-    launch_pdl(flatten_kernel, dim3(grid_for(total)), dim3(256), 0, as_stream(stream), xf, c, b, hw, x, 1);
+    launch_flatten(xf, c, b, hw, x, 1, stream);
     count_launch();
     return check_launch("flatten_kernel");
 }

@@ -1123,6 +1123,18 @@ def test_maxpool2_fwd_alignment(C, off):
     assert np.array_equal(y.cpu().numpy(), win[np.arange(len(win)), best])
 
 
+@pytest.mark.parametrize("c,b,hw", [(3, 12, 12), (2, 11, 40), (5, 33, 16), (1, 1000, 65), (4, 64, 32), (2, 70, 12),
+                                    (70000, 12, 12), (2, 9, 1)])
+def test_flatten_is_a_copy(C, c, b, hw):
+    x = torch.randn(c, b, hw, device="cuda", generator=torch.Generator("cuda").manual_seed(b))
+    xf = torch.empty(c * hw, b, device="cuda")
+    C.flatten(x, c, b, hw, xf)
+    assert torch.equal(xf.reshape(c, hw, b), x.transpose(1, 2))
+    back = torch.empty_like(x)
+    C.unflatten(xf, c, b, hw, back)
+    assert torch.equal(back, x)
+
+
 # --- failure detection: bounded waits give up and report ---------------------
 
 def test_bounded_waits_give_up_and_report(C):
