@@ -1045,8 +1045,6 @@ __device__ __forceinline__ void prox_cp_fold(const CompactArgs &a, int nrows, fl
     if (!waited && !row_mbar_wait(bar, parity)) *fail = 1;
 }
 
-__device__ __forceinline__ int nth_set_bit(uint32_t m, int k);
-__device__ __forceinline__ int warp_last_le(int pre, int e);
 
 // The kept value of the lane's entry of a 32-entry step: z - sign(z)*thr with
 // z the folded value at a stored position and fl(0 - fl(eta*G)) elsewhere.
@@ -1739,20 +1737,26 @@ __global__ void __launch_bounds__(256) tr_write_kernel(const int32_t *__restrict
 //  count: lane r loads row r's word; a 32 x 32 bit transpose (five shuffle
 //         stages) gives lane j the rows present in column 32c + j; its popcount
 //         is the block's count for that column.
-//  write: the block's kept entries are enumerated twice, 32 at a time, one
-//         entry per lane. Row-major order (the CSR order): the entry's row is
-//         found by a binary search over the rows' exclusive kept counts, its
-//         column as the k-th set bit of the row's word; its CSR position is
-//         the word position + k, so the value is read and t_pos written
-//         coalesced, and the value goes to a 32 x 32 shared tile.
-//         Column-major order (the transposed order): the same with the
-//         columns' counts and masks; consecutive entries of a column are
-//         consecutive positions of its transposed run, so t_col and t_val
-//         are written coalesced as well. A pass costs ceil(kept / 32)
-//         iterations instead of one per row (or column) of the block; a
-//         block with more than kTrbWalkMin kept entries is instead walked
-//         row by row (lane = column) and column by column (lane = row),
-//         which is cheaper once most lanes hold an entry.
+//  write: the block's kept entries are listed once in shared memory in
+//         row-major (CSR) order, lane r writing (r, j) for each set bit j of
+//         row r's word, and then handled 32 at a time, one entry per lane.
+//         The CSR position is the word position plus the rank in the row, so
+//         the value is read and t_pos written coalesced; the rank in the
+//         column (a popcount of the column's mask) gives the entry's place in
+//         column-major order, where its value and its (r, j) are staged.
+//         The staged list is the transposed order: consecutive entries of a
+//         column are consecutive positions of its run, so t_col and t_val are
+//         written coalesced as well. What bounds it is instructions: finding
+//         an entry's row by a search over the lanes and its column as the
+//         k-th set bit, in both orders, took more than half of them (prox
+//         update of 4096 x 4096 at 5%: 68.6 -> 65.0 us, kept 36%: 147.4 ->
+//         134.4 us, ADAM update of 1000 x 4096 at 20%: 59.5 -> 56.9 us).
+//         A block with more than kTrbWalkMin kept entries is instead walked
+//         row by row (lane = column) and column by column (lane = row), which
+//         is cheaper once most lanes hold an entry. Walked above 256, 384, 512,
+//         640 and 768: 4096 x 4096, 36% kept 141.4, 137.1, 133.0, 134.1, 136.4
+//         us; 51% kept 167 to 168 up to 512, then 173 and 180 us. 512 is also
+//         what the tile's 4 KB hold as two lists and the values.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) trb_count_kernel(const uint32_t *__restrict__ keepbits, int32_t rows,
                                                         int32_t wpr, int32_t cols, int32_t *__restrict__ cnt) {
@@ -1768,33 +1772,6 @@ __global__ void __launch_bounds__(256) trb_count_kernel(const uint32_t *__restri
     cnt[(int64_t)b * cols + c * 32 + lane] = __popc(colmask);
 }
 
-// Position of the k-th (from 0) set bit of m, for k < popc(m); always 0..31.
-__device__ __forceinline__ int nth_set_bit(uint32_t m, int k) {
-    int pos = 0;
-#pragma unroll
-    for (int sft = 16; sft >= 1; sft >>= 1) {
-        const int c = __popc(m & ((1u << sft) - 1u));
-        if (k >= c) {
-            k -= c;
-            m >>= sft;
-            pos += sft;
-        }
-    }
-    return pos;
-}
-
-// Largest lane r with pre(r) <= e, for pre nondecreasing over the lanes and
-// pre(0) = 0 <= e. Every lane of the warp must call it.
-__device__ __forceinline__ int warp_last_le(int pre, int e) {
-    int r = 0;
-#pragma unroll
-    for (int sft = 16; sft >= 1; sft >>= 1) {
-        const int v = __shfl_sync(0xffffffffu, pre, r + sft);
-        if (v <= e) r += sft;
-    }
-    return r;
-}
-
 __device__ __forceinline__ int warp_exclusive_sum(int x, int &total) {
     const int lane = threadIdx.x & 31;
     int inc = x;
@@ -1807,7 +1784,7 @@ __device__ __forceinline__ int warp_exclusive_sum(int x, int &total) {
     return inc - x;
 }
 
-constexpr int kTrbWalkMin = 384;   // kept entries of a 32 x 32 block above which it is walked
+constexpr int kTrbWalkMin = 512;   // kept entries of a 32 x 32 block above which it is walked
 
 __global__ void __launch_bounds__(256) trb_write_kernel(const uint32_t *__restrict__ keepbits,
                                                         const int32_t *__restrict__ wordpos, int32_t rows,
@@ -1828,7 +1805,7 @@ __global__ void __launch_bounds__(256) trb_write_kernel(const uint32_t *__restri
     const int32_t rp_mine = my_row < rows ? __ldg(wordpos + (int64_t)my_row * wpr + c) : 0;
     const int col = c * 32 + lane;
     // start of this block's part of column `col`'s transposed run
-    const int64_t cb_mine = (int64_t)__ldg(t_row_ptr + col) + __ldg(off + (int64_t)b * cols + col);
+    const int32_t cb_mine = __ldg(t_row_ptr + col) + __ldg(off + (int64_t)b * cols + col);
     const uint32_t cm_mine = warp_transpose32(rw_mine);   // lane j: the block's rows kept in column 32c + j
     int total;
     const int rpre = warp_exclusive_sum(__popc(rw_mine), total);
@@ -1874,50 +1851,48 @@ __global__ void __launch_bounds__(256) trb_write_kernel(const uint32_t *__restri
         }
         return;
     }
+    // lane r lists its row's columns: code (r, j) of entry e in CSR order
+    uint16_t *code = reinterpret_cast<uint16_t *>(tl), *tcode = code + kTrbWalkMin;
+    float *tv = reinterpret_cast<float *>(tcode + kTrbWalkMin);
+    for (uint32_t x = rw_mine, e = rpre; x; x &= x - 1, ++e) code[e] = (uint16_t)(lane * 32 + __ffs(x) - 1);
+    __syncwarp();
+    const int32_t rbase = rp_mine - rpre, cbase = cb_mine - cpre;
     constexpr int kRounds = 4;   // 32-entry rounds whose value loads are in flight together
     for (int e00 = 0; e00 < total; e00 += 32 * kRounds) {   // row-major (CSR) order
         float v[kRounds];
-        int64_t pr[kRounds], pc[kRounds];
-        int at[kRounds];
+        int at[kRounds], rj[kRounds];
 #pragma unroll
         for (int q = 0; q < kRounds; ++q) {
-            at[q] = -1;
             if (e00 + 32 * q >= total) continue;   // the same for every lane
             const int e = e00 + 32 * q + lane;
-            const int r = warp_last_le(rpre, e);
-            const uint32_t rw = __shfl_sync(0xffffffffu, rw_mine, r);
-            const int k = e - __shfl_sync(0xffffffffu, rpre, r);
-            const int32_t rp = __shfl_sync(0xffffffffu, rp_mine, r);
-            const int j = nth_set_bit(rw, k);
+            rj[q] = e < total ? code[e] : 0;
+            const int r = rj[q] >> 5, j = rj[q] & 31;
+            const int64_t pr = (int64_t)__shfl_sync(0xffffffffu, rbase, r) + e;
             const uint32_t cm = __shfl_sync(0xffffffffu, cm_mine, j);
-            const int64_t cb = __shfl_sync(0xffffffffu, cb_mine, j);
-            pr[q] = (int64_t)rp + k;
-            pc[q] = cb + __popc(cm & ((1u << r) - 1u));
-            at[q] = e < total ? r * 32 + (j ^ r) : -1;
-            v[q] = e < total && pr[q] < capacity ? __ldg(val + pr[q]) : 0.f;
+            at[q] = __shfl_sync(0xffffffffu, cpre, j) + __popc(cm & ((1u << r) - 1u));
+            const int64_t pc = (int64_t)__shfl_sync(0xffffffffu, cbase, j) + at[q];
+            v[q] = 0.f;
+            if (e < total && pr < capacity) {
+                v[q] = __ldg(val + pr);
+                if (pc < capacity) t_pos[pr] = (int32_t)pc;
+            }
         }
 #pragma unroll
         for (int q = 0; q < kRounds; ++q) {
-            if (e00 + 32 * q < total && at[q] >= 0) {
-                tl[at[q]] = v[q];
-                if (pc[q] < capacity && pr[q] < capacity) t_pos[pr[q]] = (int32_t)pc[q];
+            if (e00 + 32 * q + lane < total) {
+                tv[at[q]] = v[q];
+                tcode[at[q]] = (uint16_t)rj[q];
             }
         }
     }
     __syncwarp();
     for (int e0 = 0; e0 < total; e0 += 32) {   // column-major (transposed) order
         const int e = e0 + lane;
-        const int j = warp_last_le(cpre, e);
-        const uint32_t cm = __shfl_sync(0xffffffffu, cm_mine, j);
-        const int k = e - __shfl_sync(0xffffffffu, cpre, j);
-        const int64_t cb = __shfl_sync(0xffffffffu, cb_mine, j);
-        const int r = nth_set_bit(cm, k);
-        if (e < total) {
-            const int64_t p = cb + k;
-            if (p < capacity) {
-                t_col[p] = b * 32 + r;
-                t_val[p] = tl[r * 32 + (j ^ r)];
-            }
+        const int rj = e < total ? tcode[e] : 0;
+        const int64_t p = (int64_t)__shfl_sync(0xffffffffu, cbase, rj & 31) + e;
+        if (e < total && p < capacity) {
+            t_col[p] = b * 32 + (rj >> 5);
+            t_val[p] = tv[e];
         }
     }
 }

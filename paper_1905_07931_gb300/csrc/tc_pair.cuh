@@ -67,14 +67,6 @@ __device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, ui
         : "memory");
 }
 
-// K-major operand of 64-byte rows (32 16-bit elements), 64-byte swizzle:
-// 8-row groups 512 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_sw64(const void *p) {
-    const uint64_t addr = smem_u32(p);
-    return ((addr & 0x3FFFFull) >> 4) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 |
-           (uint64_t)4 << 61;
-}
-
 // Instruction descriptor, kind::f16 with float32 accumulators, both operands
 // K-major: type 0 = f16, 1 = bf16.
 __host__ __device__ constexpr uint32_t idesc_f16(int type, int m, int n) {

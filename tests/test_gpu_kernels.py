@@ -1135,6 +1135,45 @@ def test_flatten_is_a_copy(C, c, b, hw):
     assert torch.equal(back, x)
 
 
+@pytest.mark.parametrize("rows,counts,spare", [
+    (32, [0, 1, 511, 512, 513, 1024], 0),
+    (64, [31, 32, 33, 127, 128, 129], 0),
+    (45, [200, 512, 400, 1000], 0),       # a short last row block
+    (32, [512, 300, 600, 40], -700),      # more kept than the output holds
+])
+def test_prox_transposed_copy_blocks(C, rows, counts, spare):
+    """32 x 32 blocks with given kept counts: the transposed copy is the sorted CSR, entry by entry."""
+    rng = np.random.default_rng(rows + len(counts))
+    k = 32 * len(counts)
+    G = np.zeros((rows, k), F32)
+    for c, cnt in enumerate(counts):
+        for r0 in range(0, rows, 32):
+            h = min(32, rows - r0)
+            at = rng.permutation(h * 32)[:min(cnt, h * 32)]
+            G[r0 + at // 32, 32 * c + at % 32] = rng.choice([-1, 1], len(at)) * rng.uniform(2, 3, len(at))
+    W = C.CSR(rows, k, capacity=8, transposed=False)
+    ws = _ws(C, rows, k, 1)
+    C.csr_from_dense(torch.zeros(rows, k, device="cuda"), W, ws)
+    keep = np.argwhere(G != 0)
+    out = C.CSR(rows, k, capacity=len(keep) + spare, transposed=True)
+    out.t_val.fill_(-9.0)
+    C.prox_update_compact(W, _dev(G), 1.0, 1.0, out, ws)
+    z = -G[G != 0]
+    val = z - np.sign(z) * F32(1.0)
+    order = np.lexsort((keep[:, 0], keep[:, 1]))
+    n = len(keep)
+    pos = np.empty(n, np.int64)
+    pos[order] = np.arange(n)
+    m = n + spare if spare < 0 else n
+    fits = (np.arange(n) < m) & (pos < m)   # stored both in the CSR and in the copy
+    t_fits = fits[order][:m]
+    assert np.array_equal(out.t_pos[:m].cpu().numpy()[fits[:m]], pos[:m][fits[:m]])
+    assert np.array_equal(out.t_col_idx[:m].cpu().numpy()[t_fits], keep[order][:m, 0][t_fits])
+    assert np.array_equal(out.t_val[:m].cpu().numpy()[t_fits], val[order][:m][t_fits])
+    if spare == 0:
+        assert np.array_equal(out.t_row_ptr.cpu().numpy(), np.concatenate([[0], np.cumsum((G != 0).sum(0))]))
+
+
 # --- failure detection: bounded waits give up and report ---------------------
 
 def test_bounded_waits_give_up_and_report(C):
