@@ -166,7 +166,7 @@ def workload_config(world: int, precision: str = "tf32", prox_path: str = "fused
     """The `config` of both arms' lines: the workload and its settings."""
     return {"workload": WORKLOAD, "global_batch": BATCH * world, "per_gpu_batch": BATCH,
             "layers": list(SIZES), "densities": list(DENSITIES),
-            "weight_grad": "tf32 tcgen05" if precision == "tf32" else "fp32 simt",
+            "weight_grad": "tf32 tcgen05" if precision == "tf32" else "fp32 as bf16x3 tcgen05",
             "prox_path": prox_path if optimizer == "sgd" else "unfused", "optimizer": optimizer,
             "backward_streams": 2 if overlap == "on" else 1,
             "l2": "flushed between steps (256 MB write, outside the timed region)",
@@ -392,8 +392,8 @@ FUSED_OP_SOURCES = ["fused_prox.cu", "compact.cu", "tc_common.cuh", "common.cuh"
 # the ncu command whose CSV record_traffic reads: the ops' kernels only
 TRAFFIC_NCU = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none "
                "-k regex:'fp_oldbits|gemm_prox|fp_rowscan|fp_rows_cols|fp_two_scans|scan_clamped|scan_single|trb_|"
-               "tr_colscan|spmm_merge' "
-               "-c 60 --csv --log-file bench_dram.csv")
+               "tr_colscan|spmm_merge|spmm_tc' "
+               "-c 80 --csv --log-file bench_dram.csv")
 
 
 def record_traffic(csv_path: str, out_path: str) -> dict:
@@ -434,21 +434,31 @@ def record_traffic(csv_path: str, out_path: str) -> dict:
                      "sparse product of the classifier-head step, summed over the op's kernels (second eager step "
                      "of the run), from: " + TRAFFIC_NCU + " python bench.py --steps 1 --warmup 1 --no-cpu-baseline "
                      "--no-kernels --overlap off, then python bench.py --record-traffic bench_dram.csv (the counters "
-                     "take one pass; only the ops' kernels are captured, the first 60 launches: 4 at start-up, 28 "
+                     "take one pass; only the ops' kernels are captured, the first 80 launches: 4 at start-up, up to 33 "
                      "per step). ncu flushes the caches between kernels, so output lines still dirty in L2 when a "
                      "kernel ends are not counted: an op whose output fits in L2 shows fewer bytes than it writes."}
     # the step's sparse products, in call order: forward layers 0, 1, 2, then
     # the backward products of layers 2 and 1 (second eager step)
-    sp = [k for k in seq if "spmm_merge_kernel" in k["name"] or "spmm_group_kernel" in k["name"]]
+    # (a product that may take the tensor cores launches spmm_tc_kernel behind
+    # spmm_merge_kernel)
+    sp = []
+    for k in seq:
+        if "spmm_merge_kernel" in k["name"] or "spmm_group_kernel" in k["name"]:
+            sp.append([k])
+        elif "spmm_tc_kernel" in k["name"] and sp:
+            sp[-1].append(k)
     if len(sp) >= 10:
         labels = ["spmm_fwd_bias_act[layer 0]", "spmm_fwd_bias_act[layer 1]", "spmm_fwd_bias_act[layer 2]",
                   "spmm_bwd_t_relu[layer 2]", "spmm_bwd_t_relu[layer 1]"]
-        srcs = ["spmm.cu", "common.cuh"]
-        for lab, k in zip(labels, sp[5:10]):
-            rd, wr = k.get("dram__bytes_read.sum", 0.0), k.get("dram__bytes_write.sum", 0.0)
+        srcs = ["spmm.cu", "spmm_tc.cu", "spmm_tc.cuh", "tc_pair.cuh", "common.cuh"]
+        for lab, call in zip(labels, sp[5:10]):
+            rd = sum(k.get("dram__bytes_read.sum", 0.0) for k in call)
+            wr = sum(k.get("dram__bytes_write.sum", 0.0) for k in call)
+            us = sum(k.get("gpu__time_duration.sum", 0.0) for k in call) / 1e3
             pending[lab] = {"dram_bytes_per_call": int(rd + wr), "dram_read": int(rd), "dram_write": int(wr),
-                            "ncu_us_serialised": round(k.get("gpu__time_duration.sum", 0.0) / 1e3, 1),
-                            "kernels": [k["name"].split("(")[0].replace("csrt::", "").replace("void ", "")],
+                            "ncu_us_serialised": round(us, 1),
+                            "kernels": [k["name"].split("(")[0].replace("csrt::", "").replace("void ", "")
+                                        for k in call],
                             "sources": srcs, "sha256_16": source_digest(srcs)}
     for layer, call in zip((2, 1, 0), calls[3:6]):
         rd = sum(k.get("dram__bytes_read.sum", 0.0) for k in call)
@@ -683,12 +693,14 @@ def main():
                       "peak_source": "measured FP32 FMA rate (library probe, fma_peak_kernel)"})
     if dom["name"] in ("weight_grad_dense", "weight_grad_prox_update") and dom["info"].get("n") \
             and args.precision == "fp32":
-        # --precision fp32: the contraction runs on the FP32 CUDA cores
+        # --precision fp32: each factor as the sum of three bf16 parts, six
+        # products of the parts on the tensor cores; algorithmic flops 2MKN
+        # against a sixth of the measured bf16 rate
         flops = 2.0 * dom["info"]["M"] * dom["info"]["K"] * dom["info"]["n"]
-        peak = C.fma_peak_tflops()
-        cands.append({"bound": "alu", "achieved": round(flops / t_s / 1e12, 2), "peak": round(peak, 1),
+        peak = peaks["bf16_tflops"] / 6
+        cands.append({"bound": "tensor", "achieved": round(flops / t_s / 1e12, 2), "peak": round(peak, 1),
                       "unit": "TFLOP/s", "frac": round(flops / t_s / 1e12 / peak, 4),
-                      "peak_source": "measured FP32 FMA rate (library probe, fma_peak_kernel)"})
+                      "peak_source": f"bf16_tflops / 6 ({peak_kind} peaks)"})
     elif dom["name"] in ("weight_grad_dense", "weight_grad_prox_update") and dom["info"].get("n"):
         # a TF32 contraction: its peak is the cuBLAS TF32 rate measured here (the
         # measured bf16 rate x the nominal tf32/bf16 ratio 1.1/2.25 beside it);
@@ -709,7 +721,8 @@ def main():
         same_kernels = dom["name"] in ("spmm_fwd", "spmm_bwd_t", "spmm_fwd_bias_act", "spmm_bwd_t_relu") or (
             args.precision == "tf32" and args.prox_path == "fused" and args.optimizer == "sgd")
         if args.precision == "fp32" and dom["name"] == "weight_grad_prox_update":
-            kernel = "gemm_nt_f32_kernel + prox_count_kernel + prox_place_kernel (the op's unfused route at FP32)"
+            kernel = ("split_rows_kernel + gemm_split_kernel + prox_count_kernel + prox_place_kernel "
+                      "(the op's unfused route at FP32)")
         roof.update({"traffic": recorded_traffic(dom["label"]) if same_kernels else None, "kernel": kernel,
                      "op": dom["label"],
                      "algorithmic_bytes": int(bytes_) if bytes_ else None, "launch_ms": round(dom["ms"], 4)})
@@ -784,9 +797,9 @@ def profile_ops(net, C, torch, eta, lam, flush):
     names = ["spmm_fwd", "spmm_bwd_t", "spmm_fwd_bias_act", "spmm_bwd_t_relu", "weight_grad_dense",
              "weight_grad_sddmm", "prox_update_compact", "prox_rmsprop_update_compact", "prox_adam_update_compact",
              "weight_grad_prox_update", "debias_update", "bias_act_fwd", "relu_bwd", "bias_grad_sgd", "softmax_xent"]
-    kernel_of = {"spmm_fwd": "spmm_merge_kernel", "spmm_bwd_t": "spmm_merge_kernel",
+    kernel_of = {"spmm_fwd": "spmm_merge_kernel", "spmm_bwd_t": "spmm_merge_kernel",  # and spmm_tc_kernel, dense layers
                  "spmm_fwd_bias_act": "spmm_merge_kernel", "spmm_bwd_t_relu": "spmm_merge_kernel",
-                 "weight_grad_dense": "gemm_tf32_tc_persistent_kernel", "weight_grad_sddmm": "sddmm_kernel",
+                 "weight_grad_dense": "gemm_tf32_tc_persistent_kernel", "weight_grad_sddmm": "sddmm_wide_kernel",
                  "prox_update_compact": "prox_count_kernel", "prox_rmsprop_update_compact": "prox_rows_kernel",
                  "prox_adam_update_compact": "prox_rows_kernel", "weight_grad_prox_update": "gemm_prox_tc_kernel",
                  "debias_update": "debias_kernel"}
