@@ -154,13 +154,13 @@ __device__ __forceinline__ void st_write(const StArgs &a, int tile, uint32_t ran
     }
 }
 
-// Counting in at a cut tile. cnt[0]: the parts that are there (bits 0-7) and
-// the shares whose pairs gave up waiting (from bit 8); cnt[1]: the pairs that
-// are through, the last of which zeroes both.
+// Counting in at a cut tile: the parts that are there (bits 0-7) and the
+// shares whose pairs gave up waiting (from bit 8). The first kernel of every
+// product zeroes the counters.
 constexpr uint32_t kStPartsMask = 0xff;
 
-// One pair's part in adding up a cut tile; `seen` is what cnt[0] was when it
-// counted in.
+// One pair's part in adding up a cut tile; `seen` is what its counter was when
+// it counted in.
 template <int kN>
 __device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, int tile, uint32_t rank, int q, int h,
                                       int tid, uint32_t seen, volatile uint32_t *state) {
@@ -169,7 +169,7 @@ __device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, 
     const int p0 = st_pair_of(units, a.pairs, t0), parts = st_pair_of(units, a.pairs, t0 + a.chunks - 1) - p0 + 1;
     // (the pair that begins a tile has ended another, whose share it does)
     const int shares = imin(parts - 1, kUnits), own = pair - p0 - 1;
-    uint32_t *cnt = a.cnt + 2 * (tile * 2 + (int)rank);
+    uint32_t *cnt = a.cnt + (tile * 2 + (int)rank);
     if (tid == 0) {
         uint32_t todo = own >= 0 && own < shares ? 1u << own : 0u;
         if ((int)(seen & kStPartsMask) == parts - 1) {
@@ -215,7 +215,6 @@ __device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, 
             st_write<kN>(a, tile, rank, q, h * (kN / 4) + c * 8, v, wsc);
         }
     }
-    if (tid == 0 && (int)atomicAdd(cnt + 1, 1u) == parts - 1) cnt[0] = cnt[1] = 0;
 }
 
 template <int kN>
@@ -447,7 +446,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
             __threadfence();
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kStEpiWarps) : "memory");
             if (tid == 0) {
-                const uint32_t seen = atomicAdd(a.cnt + 2 * (tile * 2 + (int)rank), 1u);
+                const uint32_t seen = atomicAdd(a.cnt + (tile * 2 + (int)rank), 1u);
                 if (begins) seen_b = seen;
                 else seen_e = seen;
             }
@@ -488,9 +487,11 @@ static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int64_t capacity, int
     const int64_t chunks = ceil_div(k, kStChunk);
     return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)4 * n * st_ld(k)) +
            st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) + st_align((size_t)4 * rows) +
-           st_align((size_t)4 * chunks * ceil_div(n, n_tile / 4)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
+           st_align((size_t)4 * chunks * ceil_div(n, n_tile / 4)) +
+           st_align((size_t)8 * ceil_div(rows, 256) * ceil_div(n, n_tile)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
 }
 constexpr int32_t kStMinRows = 256, kStMinK = 1024, kStMinN = 65;
+constexpr int32_t kStMaxTiles = 4096;
 static bool st_shape_ok(int32_t rows, int32_t k) {
     return rows >= kStMinRows && k >= kStMinK && k <= kTcMaxChunks * kStChunk;
 }
@@ -514,8 +515,8 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     const int chunks = ceil_div(k, kStChunk);
     plan->n_tile = n_tile;
     plan->tiles_n = ceil_div(n, n_tile);
+    if ((int64_t)ceil_div(rows, 256) * plan->tiles_n > kStMaxTiles) return;
     plan->tiles = ceil_div(rows, 256) * plan->tiles_n;
-    if (4 * plan->tiles > (int)kWsCounterInts) return;
     const int64_t units = (int64_t)plan->tiles * chunks;
     // Whole tiles per pair where that costs no more than cutting them
     // (microseconds; the partial sums take 4 us and 2.2 us for each eighth of
@@ -559,8 +560,9 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)));
     plan->prep.wscale = reinterpret_cast<float *>(take((size_t)4 * rows));
     plan->prep.xscale = reinterpret_cast<float *>(take((size_t)4 * chunks * ceil_div(n, n_tile / 4)));
+    plan->prep.counters = 2 * plan->tiles;
+    plan->prep.cnt = reinterpret_cast<uint32_t *>(take((size_t)4 * plan->prep.counters));
     plan->partial = reinterpret_cast<float *>(p);
-    plan->cnt = ws_counters(ws);
     plan->prep.k = k;
     plan->prep.ld = st_ld(k);
     plan->prep.chunks = chunks;
@@ -601,7 +603,7 @@ int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t
     a.xscale = plan.prep.xscale;
     a.y = y;
     a.partial = plan.partial;
-    a.cnt = reinterpret_cast<uint32_t *>(plan.cnt);
+    a.cnt = plan.prep.cnt;
     a.bias = bias;
     a.mask = mask;
     a.relu = relu;

@@ -27,12 +27,13 @@ struct SpmmTcPrep {
     float *xscale;       // [chunks][ceil(n / width)] undoes that (NaN likewise)
     int32_t k, ld, chunks, width;
     int32_t vec;         // rows of X may be read as float4
+    uint32_t *cnt;       // [counters] of the tensor-core kernel's cut tiles, zeroed here: a kernel that gave up
+    int32_t counters;    // waiting leaves nothing behind for the next call
 };
 
 struct SpmmTcPlan {
     SpmmTcPrep prep;
     float *partial;
-    int32_t *cnt;
     int32_t n_tile, tiles_n, tiles, pairs;
     bool whole;   // no tile is shared by pairs
 };
@@ -274,6 +275,7 @@ __device__ __forceinline__ void spmm_tc_prep(const SpmmTcPrep &a, const int32_t 
     const int nb = (n + a.width - 1) / a.width;
     const int ws = (rows + kTcGroup - 1) / kTcGroup, xs = a.chunks * nb;
     const int grid = (int)gridDim.x, b = (int)blockIdx.x;
+    for (int i = b * blockDim.x + threadIdx.x; i < a.counters; i += grid * blockDim.x) a.cnt[i] = 0;
     for (int i = b; i < ws; i += grid) spmm_tc_prep_w(a, row_ptr, col, val, rows, i, s_tab);
     // X by the blocks that had fewer groups to do
     const int busy = ws % grid, idle = grid - busy;

@@ -1,0 +1,59 @@
+"""The tensor-core paths (dense sparse-matrix products, float32 gradient) where their operands, their workspace or the
+host's state are not the ordinary ones: each compared with plain torch in 64 bits or with the same call on a fresh
+workspace."""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -24
+
+
+@pytest.fixture(scope="module")
+def C():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1905_07931_gb300 import csrtrain
+    csrtrain.lib()
+    return csrtrain
+
+
+def _gen(seed):
+    return torch.Generator("cuda").manual_seed(seed)
+
+
+def _weights(m, k, density, seed):
+    g = _gen(seed)
+    w = torch.randn(m, k, device="cuda", generator=g)
+    return w * (torch.rand(m, k, device="cuda", generator=g) < density)
+
+
+def _csr(C, dense, ws, transposed=False, capacity=None):
+    w = C.CSR(*dense.shape, capacity=capacity, transposed=transposed)
+    C.csr_from_dense(dense.contiguous(), w, ws)
+    return w
+
+
+def _bits(t):
+    return t.view(torch.int32)
+
+
+@pytest.mark.parametrize("m,k,n", [(777, 4000, 333), (1300, 5000, 99)])   # column tiles of 256 and 128, all shared
+def test_product_after_a_wait_that_gave_up(C, m, k, n):
+    """A kernel that gives up waiting leaves counters behind; the status is cleared, the next product is right."""
+    ws = C.Workspace(m, k, n)
+    dense = _weights(m, k, 0.3, m)
+    w = _csr(C, dense, ws)
+    x = torch.randn(k, n, device="cuda", generator=_gen(n))
+    want, got = (torch.full((m, n), float("nan"), device="cuda") for _ in range(2))
+    C.launch_count(reset=True)
+    C.spmm_fwd(w, x, want, ws)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    words = ws.buf[256:].view(torch.int32)
+    for stale in (1, 0x101, 7):
+        words.fill_(stale)           # counters and scratch alike
+        ws.clear_status()
+        C.spmm_fwd(w, x, got, ws)
+        assert torch.equal(_bits(got), _bits(want))
+    assert ws.status()[0] == 0
