@@ -2,11 +2,15 @@
 host's state are not the ordinary ones: each compared with plain torch in 64 bits or with the same call on a fresh
 workspace."""
 
-import numpy as np
+import os
+import subprocess
+import sys
+
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 U = 2.0 ** -24
 
 
@@ -57,3 +61,34 @@ def test_product_after_a_wait_that_gave_up(C, m, k, n):
         C.spmm_fwd(w, x, got, ws)
         assert torch.equal(_bits(got), _bits(want))
     assert ws.status()[0] == 0
+
+
+FIRST_CALLS = """
+import threading, torch
+from paper_1905_07931_gb300 import csrtrain as C
+N, m, n = 24, 512, 256
+g = torch.Generator("cuda").manual_seed(1)
+dy, x = (torch.randn(m, n, device="cuda", generator=g) for _ in range(2))
+ws = [C.Workspace(m, m, n) for _ in range(N + 1)]
+out = [torch.zeros(m, m, device="cuda") for _ in range(N + 1)]
+torch.cuda.synchronize()
+launches, gate = [None] * N, threading.Barrier(N)
+def call(i):
+    torch.cuda.set_device(0)
+    gate.wait()
+    C.weight_grad_dense(dy, x, out[i], ws[i], precision=0)
+    launches[i] = C.launch_count()
+threads = [threading.Thread(target=call, args=(i,)) for i in range(N)]
+[t.start() for t in threads]
+[t.join() for t in threads]
+C.weight_grad_dense(dy, x, out[N], ws[N], precision=0)
+torch.cuda.synchronize()
+assert launches == [2] * N, launches      # the tensor-core path in every thread
+assert all(torch.equal(o, out[N]) for o in out)
+"""
+
+
+def test_first_calls_of_many_threads(C):
+    """A process whose first calls come from many threads at once takes the same path in all of them."""
+    r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
