@@ -41,6 +41,8 @@
 // Values a factor can't take here (2^50 and more, infinities, NaN) turn the
 // scale of their row or chunk into NaN, which ends as a NaN in the sums they
 // touch; such entries of Y are computed again from the CSR row.
+#include <atomic>
+
 #include "spmm_tc.cuh"
 #include "tc_pair.cuh"
 
@@ -505,6 +507,22 @@ size_t spmm_tc_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
     return imax(f, b) <= (size_t)1 << 30 ? imax(f, b) : 0;   // beyond a gigabyte: the sparse kernel alone
 }
 
+// The kernel may use its shared memory (asked once per device).
+static bool st_kernel_ready() {
+    static std::atomic<int> state[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (state[dev].load() == 0) {
+        const bool ok = cudaFuncSetAttribute(spmm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             st_smem<256>()) == cudaSuccess &&
+                        cudaFuncSetAttribute(spmm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             st_smem<128>()) == cudaSuccess;
+        if (!ok) cudaGetLastError();
+        state[dev].store(ok ? 1 : 2);
+    }
+    return state[dev].load() == 1;
+}
+
 void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const float *x, void *ws, size_t ws_bytes,
                   int32_t sparse_units, double t_entry, SpmmTcPlan *plan) {
     plan->prep.nnz_min = 0;
@@ -568,32 +586,20 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.chunks = chunks;
     plan->prep.width = n_tile / 4;
     plan->prep.vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    if (!make_map16(&plan->map_x, plan->prep.xp, false, (int64_t)2 * n, k, plan->prep.ld, n_tile / 2, kStChunk)) return;
+    if (!st_kernel_ready()) return;
     plan->prep.nnz_min = nnz_min;
 }
 
 int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t *col, const float *val, int32_t rows,
                    const float *x, int32_t n, float *y, const float *bias, int32_t relu, const float *mask, void *ws,
                    cudaStream_t s) {
-    CUtensorMap mx;
-    const int32_t k = plan.prep.k;
-    if (!make_map16(&mx, plan.prep.xp, false, (int64_t)2 * n, k, plan.prep.ld, plan.n_tile / 2, kStChunk))
-        return fail(CSRT_ERR_CUDA, "spmm: the tensor map of X's planes could not be made");
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    CSRT_CHECK_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        CSRT_CHECK_CUDA(cudaFuncSetAttribute(spmm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             st_smem<256>()));
-        CSRT_CHECK_CUDA(cudaFuncSetAttribute(spmm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             st_smem<128>()));
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
     StArgs a;
     a.row_ptr = row_ptr;
     a.col = col;
     a.val = val;
     a.rows = rows;
-    a.k = k;
+    a.k = plan.prep.k;
     a.n = n;
     a.parts = plan.prep.parts;
     a.place = plan.prep.place;
@@ -615,8 +621,8 @@ int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t
     a.whole = plan.whole;
     a.hdr = static_cast<WsHeader *>(ws);
     const unsigned grid = (unsigned)(2 * plan.pairs);
-    if (plan.n_tile == 256) launch_pair(spmm_tc_kernel<256>, grid, kStThreads, st_smem<256>(), s, mx, a);
-    else launch_pair(spmm_tc_kernel<128>, grid, kStThreads, st_smem<128>(), s, mx, a);
+    if (plan.n_tile == 256) launch_pair(spmm_tc_kernel<256>, grid, kStThreads, st_smem<256>(), s, plan.map_x, a);
+    else launch_pair(spmm_tc_kernel<128>, grid, kStThreads, st_smem<128>(), s, plan.map_x, a);
     count_launch();
     return check_launch("spmm_tc_kernel");
 }

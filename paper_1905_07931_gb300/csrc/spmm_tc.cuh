@@ -4,6 +4,7 @@
 // in which the GEMM expands them.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_fp16.h>
 
 #include "common.cuh"
@@ -33,6 +34,7 @@ struct SpmmTcPrep {
 
 struct SpmmTcPlan {
     SpmmTcPrep prep;
+    CUtensorMap map_x;   // of prep.xp
     float *partial;
     int32_t n_tile, tiles_n, tiles, pairs;
     bool whole;   // no tile is shared by pairs
@@ -40,6 +42,8 @@ struct SpmmTcPlan {
 
 size_t spmm_tc_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n);
 // Fills the plan (prep.nnz_min > 0) if the product may run on the tensor cores.
+// Everything that can fail is done here, before the product's first kernel is
+// enqueued: a product that can't be planned runs on the sparse kernels alone.
 // `units` and `t_entry` describe the sparse kernel: the work units its rows and
 // entries are cut into, and its time per entry (microseconds).
 void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const float *x, void *ws, size_t ws_bytes,
