@@ -52,10 +52,12 @@ constexpr int kGsEpiWarps = 16;                        // per TMEM lane quarter 
 constexpr int kGsEpiCols = 64;
 constexpr int kGsProd = 4;                             // a warpgroup of producers (TMA, MMA, two idle)
 constexpr int kGsThreads = 32 * (kGsProd + kGsEpiWarps);
-// register split within the launch's 640 x 96: the sums (64), a block read
-// back (32) and addresses need more than 96 in the epilogue warps
+// register split (ptxas gives the launch 640 x 96; it is found to hold the
+// shares before it is used): the sums (64), a block read back (32) and
+// addresses need more than 96 in the epilogue warps
 constexpr int kGsProdRegs = 32, kGsEpiRegs = 112;
-static_assert(128 * kGsProdRegs + 32 * kGsEpiWarps * kGsEpiRegs <= kGsThreads * 96, "register split");
+constexpr int kGsSplitRegs = 128 * kGsProdRegs + 32 * kGsEpiWarps * kGsEpiRegs;
+static_assert(kGsSplitRegs <= kGsThreads * 96, "register split");
 constexpr int kGsTile = 256;
 constexpr int kGsStageOut = 32 * 16 * 4;               // a 32 x 16 block on its way out
 constexpr int kGsSmem = kGsStages * kGsStageBytes + kGsEpiWarps * kGsStageOut + 1024 + 256;
@@ -391,14 +393,8 @@ int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_
     if (!make_map16(&ma, pdy, true, (int64_t)3 * m, n, ld, 128, kGsStageCols) ||
         !make_map16(&mb, px, true, (int64_t)3 * k, n, ld, 128, kGsStageCols))
         return CSRT_OK;
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    CSRT_CHECK_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return CSRT_OK;
-    if (!attr_set[dev]) {
-        CSRT_CHECK_CUDA(cudaFuncSetAttribute(gemm_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGsSmem));
-        attr_set[dev] = true;
-    }
+    static std::atomic<int> ready[64];
+    if (!pair_kernel_ready(gemm_split_kernel, ready, kGsSmem, kGsThreads, kGsSplitRegs)) return CSRT_OK;
     GsArgs a;
     a.g = g;
     a.m = m;

@@ -41,8 +41,6 @@
 // Values a factor can't take here (2^50 and more, infinities, NaN) turn the
 // scale of their row or chunk into NaN, which ends as a NaN in the sums they
 // touch; such entries of Y are computed again from the CSR row.
-#include <atomic>
-
 #include "spmm_tc.cuh"
 #include "tc_pair.cuh"
 
@@ -50,12 +48,14 @@ namespace csrt {
 
 constexpr int kStChunk = kTcChunk;
 // Warps: 0 TMA, 1 MMA (2 and 3 idle), eight that expand W (a group of 16 rows
-// each), sixteen that add up and write; registers within the launch's 896 x 72.
+// each), sixteen that add up and write. kStSplitRegs: what their shares come to
+// (the launch is found to hold them before it is used; ptxas gives 896 x 72).
 constexpr int kStExpandWarps = 8, kStEpiWarps = 16;
 constexpr int kStThreads = 32 * (4 + kStExpandWarps + kStEpiWarps);
 constexpr int kStProdRegs = 32, kStExpandRegs = 40, kStEpiRegs = 96;
-static_assert(128 * kStProdRegs + 32 * (kStExpandWarps * kStExpandRegs + kStEpiWarps * kStEpiRegs) <= kStThreads * 72,
-              "register split");
+constexpr int kStSplitRegs =
+    128 * kStProdRegs + 32 * (kStExpandWarps * kStExpandRegs + kStEpiWarps * kStEpiRegs);
+static_assert(kStSplitRegs <= kStThreads * 72, "register split");
 constexpr int kStASlice = 128 * kStChunk * 2;
 template <int kN> __host__ __device__ constexpr int st_bslice() { return kN / 2 * kStChunk * 2; }
 template <int kN> __host__ __device__ constexpr int st_stage() { return 2 * (kStASlice + st_bslice<kN>()); }
@@ -507,22 +507,6 @@ size_t spmm_tc_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
     return imax(f, b) <= (size_t)1 << 30 ? imax(f, b) : 0;   // beyond a gigabyte: the sparse kernel alone
 }
 
-// The kernel may use its shared memory (asked once per device).
-static bool st_kernel_ready() {
-    static std::atomic<int> state[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-    if (state[dev].load() == 0) {
-        const bool ok = cudaFuncSetAttribute(spmm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             st_smem<256>()) == cudaSuccess &&
-                        cudaFuncSetAttribute(spmm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             st_smem<128>()) == cudaSuccess;
-        if (!ok) cudaGetLastError();
-        state[dev].store(ok ? 1 : 2);
-    }
-    return state[dev].load() == 1;
-}
-
 void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const float *x, void *ws, size_t ws_bytes,
                   int32_t sparse_units, double t_entry, SpmmTcPlan *plan) {
     plan->prep.nnz_min = 0;
@@ -587,7 +571,10 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.width = n_tile / 4;
     plan->prep.vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
     if (!make_map16(&plan->map_x, plan->prep.xp, false, (int64_t)2 * n, k, plan->prep.ld, n_tile / 2, kStChunk)) return;
-    if (!st_kernel_ready()) return;
+    static std::atomic<int> ready256[64], ready128[64];
+    if (!(n_tile == 256 ? pair_kernel_ready(spmm_tc_kernel<256>, ready256, st_smem<256>(), kStThreads, kStSplitRegs)
+                        : pair_kernel_ready(spmm_tc_kernel<128>, ready128, st_smem<128>(), kStThreads, kStSplitRegs)))
+        return;
     plan->prep.nnz_min = nnz_min;
 }
 

@@ -11,6 +11,8 @@
 // barriers of both CTAs.
 #pragma once
 
+#include <atomic>
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -115,6 +117,29 @@ inline bool make_map16(CUtensorMap *map, const void *base, bool bf16, int64_t ro
                     box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
+}
+
+// Whether this build's kernel can run on the current device as written: it may
+// use `smem` bytes of shared memory, and its launches of `threads` threads hold
+// `regs` registers, the sum of what its warps lower and raise their shares to
+// (setmaxnreg.inc waits without a bound for registers the launch does not
+// hold; how many it holds is the compiler's choice). `state`: 64 zeros, one per
+// device, asked once.
+template <typename K>
+inline bool pair_kernel_ready(K kernel, std::atomic<int> *state, int smem, int threads, int regs) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    int known = state[dev].load();
+    if (known == 0) {
+        cudaFuncAttributes fa{};
+        const bool ok =
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+            cudaFuncGetAttributes(&fa, kernel) == cudaSuccess && fa.numRegs * threads >= regs;
+        if (!ok) cudaGetLastError();   // (not an error of the call: it takes the other path)
+        known = ok ? 1 : 2;
+        state[dev].store(known);
+    }
+    return known == 1;
 }
 
 // Launch of a kernel on CTA pairs (grid a multiple of 2) with programmatic
