@@ -40,7 +40,8 @@
 //
 // Values a factor can't take here (2^50 and more, infinities, NaN) turn the
 // scale of their row or chunk into NaN, which ends as a NaN in the sums they
-// touch; such entries of Y are computed again from the CSR row.
+// touch; such entries of Y are computed again from the CSR row. Rows out of
+// order or with an entry twice make the whole product run by gathering.
 #include "spmm_tc.cuh"
 #include "tc_pair.cuh"
 
@@ -73,11 +74,14 @@ struct StArgs {
     const float *x, *wscale, *xscale;
     float *y, *partial;
     uint32_t *cnt;
+    const uint8_t *marks;
+    int32_t num_marks;
     const float *bias, *mask;
     int32_t relu;
     int64_t nnz_min;
     int32_t tiles_n, tiles, chunks, pairs;
     int32_t whole;   // pairs take whole tiles
+    int32_t vec;     // rows of X may be read as float4
     WsHeader *hdr;
 };
 
@@ -107,6 +111,54 @@ __device__ __forceinline__ float st_finish(const StArgs &a, int64_t row, int64_t
     if (a.relu) v = fmaxf(v, 0.f);
     if (a.mask && !(__ldg(a.mask + row * a.n + c) > 0.f)) v = 0.f;
     return v;
+}
+
+// The whole product by gathering, for operands that the tensor cores can't take
+// (marked by the first kernel): a warp per row and 32 VW columns, which lie VW
+// to a lane; the row's entries in their order, one chain of multiply-adds per
+// element of Y.
+template <int VW>
+static __device__ __noinline__ void st_gather(const StArgs &a) {
+    const int lane = threadIdx.x & 31;
+    const int tiles = (a.n + 32 * VW - 1) / (32 * VW);
+    const int64_t work = (int64_t)a.rows * tiles, step = (int64_t)gridDim.x * (kStThreads / 32);
+    for (int64_t i = (int64_t)blockIdx.x * (kStThreads / 32) + (threadIdx.x >> 5); i < work; i += step) {
+        const int64_t row = i / tiles;
+        const int c = (int)(i % tiles) * 32 * VW + lane * VW;   // (a multiple of VW in n: all of a lane's or none)
+        const bool on = c < a.n;
+        float sum[VW] = {};
+        const int32_t end = __ldg(a.row_ptr + row + 1);
+        for (int32_t e0 = __ldg(a.row_ptr + row); e0 < end; e0 += 32) {
+            const int32_t cnt = min(32, end - e0);
+            const int32_t col = lane < cnt ? __ldg(a.col + e0 + lane) : 0;
+            const float val = lane < cnt ? __ldg(a.val + e0 + lane) : 0.f;
+            for (int e = 0; e < cnt; e += 8) {
+                float x[8][VW];
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {   // eight rows of X in flight
+                    const int64_t j = __shfl_sync(0xffffffffu, col, e + o);
+                    const float *p = a.x + j * a.n + c;
+                    if (e + o >= cnt || !on) continue;
+                    if constexpr (VW == 4) {
+                        const float4 v = ldg_f4(p);
+                        x[o][0] = v.x; x[o][1] = v.y; x[o][2] = v.z; x[o][3] = v.w;
+                    } else {
+                        x[o][0] = __ldg(p);
+                    }
+                }
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {
+                    const float w = __shfl_sync(0xffffffffu, val, e + o);
+                    if (e + o >= cnt || !on) continue;
+#pragma unroll
+                    for (int v = 0; v < VW; ++v) sum[v] = fmaf(w, x[o][v], sum[v]);
+                }
+            }
+        }
+        if (!on) continue;
+#pragma unroll
+        for (int v = 0; v < VW; ++v) a.y[row * a.n + c + v] = st_finish(a, row, c + v, sum[v]);
+    }
 }
 
 // First unit of pair p, and the pair that unit u belongs to.
@@ -275,8 +327,14 @@ __global__ void __launch_bounds__(kStThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
     pdl_enter();   // the operands are complete from here on
+    bool marked = false;
+    for (int i = threadIdx.x; i < a.num_marks; i += kStThreads) marked |= a.marks[i] != 0;
+    marked = __syncthreads_or(marked);   // the same for every CTA
 
-    if (warp < 4) {
+    if (marked) {
+        if (a.vec) st_gather<4>(a);
+        else st_gather<1>(a);
+    } else if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kStProdRegs));
         if (warp == 0 && lane == 0) {
             int it = 0;
@@ -490,6 +548,7 @@ static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int64_t capacity, int
     return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)4 * n * st_ld(k)) +
            st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) + st_align((size_t)4 * rows) +
            st_align((size_t)4 * chunks * ceil_div(n, n_tile / 4)) +
+           st_align((size_t)ceil_div(rows, kTcGroup)) +
            st_align((size_t)8 * ceil_div(rows, 256) * ceil_div(n, n_tile)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
 }
 constexpr int32_t kStMinRows = 256, kStMinK = 1024, kStMinN = 65;
@@ -562,6 +621,8 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)));
     plan->prep.wscale = reinterpret_cast<float *>(take((size_t)4 * rows));
     plan->prep.xscale = reinterpret_cast<float *>(take((size_t)4 * chunks * ceil_div(n, n_tile / 4)));
+    plan->prep.num_marks = ceil_div(rows, kTcGroup);
+    plan->prep.marks = reinterpret_cast<uint8_t *>(take((size_t)plan->prep.num_marks));
     plan->prep.counters = 2 * plan->tiles;
     plan->prep.cnt = reinterpret_cast<uint32_t *>(take((size_t)4 * plan->prep.counters));
     plan->partial = reinterpret_cast<float *>(p);
@@ -597,6 +658,9 @@ int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t
     a.y = y;
     a.partial = plan.partial;
     a.cnt = plan.prep.cnt;
+    a.marks = plan.prep.marks;
+    a.num_marks = plan.prep.num_marks;
+    a.vec = plan.prep.vec;
     a.bias = bias;
     a.mask = mask;
     a.relu = relu;

@@ -14,6 +14,7 @@ namespace csrt {
 constexpr int kTcChunk = 64;        // columns of W (features) per step of the GEMM
 constexpr int kTcGroup = 16;        // rows whose entries of a chunk lie together
 constexpr int kTcMaxChunks = 256;
+constexpr int32_t kTcNoColumn = 0x7fffffff;   // past the end of a row
 
 // What the first kernel of an eligible product needs: if the matrix holds at
 // least nnz_min entries it prepares both operands for the tensor-core kernel
@@ -28,6 +29,8 @@ struct SpmmTcPrep {
     float *xscale;       // [chunks][ceil(n / width)] undoes that (NaN likewise)
     int32_t k, ld, chunks, width;
     int32_t vec;         // rows of X may be read as float4
+    uint8_t *marks;      // [groups] 1: the group holds rows that the tensor cores can't take
+    int32_t num_marks;
     uint32_t *cnt;       // [counters] of the tensor-core kernel's cut tiles, zeroed here: a kernel that gave up
     int32_t counters;    // waiting leaves nothing behind for the next call
 };
@@ -140,6 +143,9 @@ __device__ __forceinline__ void spmm_tc_prep_x(const SpmmTcPrep &a, const float 
 // each chunk, added up, give every run its place, kept as the difference
 // from its place in the CSR; the second pass splits the entries and stores
 // them. tab: [chunks + 1][17] words (17: rows of one chunk in different banks).
+// Rows whose columns don't ascend have no such runs, and of two entries of one
+// column the operand could hold only one: their group is marked and left (the
+// sparse kernels, which add up whatever a row stores, take any order).
 __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_t *__restrict__ row_ptr,
                                                const int32_t *__restrict__ col, const float *__restrict__ val,
                                                int32_t rows, int32_t group, int32_t (*tab)[17]) {
@@ -162,12 +168,13 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 const int32_t i = beg[q] + i0 + h * 32 + lane;
-                c[q][h] = i < end[q] ? __ldg(col + i) : 0x7fffffff;
+                c[q][h] = i < end[q] ? __ldg(col + i) : kTcNoColumn;
                 w[q][h] = i < end[q] ? __ldg(val + i) : 0.f;
             }
     };
     uint32_t mx[2] = {0, 0};
-    int before[2] = {-1, -1};   // chunk of the entry before this step's
+    int before[2] = {-1, -1};   // column of the entry before this step's
+    bool unfit = false;
     load(0);
     // (one step more than entries need ends every row: the chunks after its
     // last entry begin at its end)
@@ -177,7 +184,7 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
         for (int q = 0; q < 2; ++q)
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
-                cc[q][h] = min(c[q][h] >> 6, a.chunks);
+                cc[q][h] = c[q][h];
                 mx[q] = max(mx[q], __float_as_uint(w[q][h]) & 0x7fffffffu);
             }
         if (i0 + 128 <= len) load(i0 + 128);
@@ -187,7 +194,10 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
             for (int h = 0; h < 4; ++h) {
                 int prev = __shfl_up_sync(0xffffffffu, cc[q][h], 1);
                 if (lane == 0) prev = before[q];
-                for (int ch = prev + 1; ch <= cc[q][h]; ++ch)   // mostly none or one
+                unfit |= cc[q][h] != kTcNoColumn && (cc[q][h] <= prev || cc[q][h] >= a.k);
+                // mostly none or one (columns before `prev`: none)
+                const int last = min(cc[q][h] >> 6, a.chunks);
+                for (int ch = max(prev >> 6, -1) + 1; ch <= last; ++ch)
                     tab[ch][warp * 2 + q] = min(i0 + h * 32 + lane, end[q] - beg[q]);
                 before[q] = __shfl_sync(0xffffffffu, cc[q][h], 31);
             }
@@ -206,7 +216,9 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
     }
     __shared__ int32_t s_sum[9];
     const int32_t base = __ldg(row_ptr + group * kTcGroup);
-    __syncthreads();
+    unfit = __syncthreads_or(unfit);
+    if (threadIdx.x == 0) a.marks[group] = unfit;
+    if (unfit) return;
     // thread = chunk: its rows' counts, the chunks' first entries by a block scan
     {
         const int ch = threadIdx.x;
@@ -258,7 +270,7 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
         for (int q = 0; q < 2; ++q)
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
-                if (cc[q][h] == 0x7fffffff) continue;
+                if (cc[q][h] == kTcNoColumn) continue;
                 __half hi, lo;
                 fp16_split(ww[q][h] * down[q], hi, lo);
                 const int32_t p = tab[cc[q][h] >> 6][warp * 2 + q] + i0 + h * 32 + lane;

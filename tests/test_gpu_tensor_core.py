@@ -92,3 +92,32 @@ def test_first_calls_of_many_threads(C):
     """A process whose first calls come from many threads at once takes the same path in all of them."""
     r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("n", [256, 333])
+@pytest.mark.parametrize("how", ["reversed", "shuffled", "twice"])
+def test_product_of_rows_in_any_order(C, n, how):
+    """Rows whose columns don't ascend, or that hold an entry of one column twice, are added up as they are stored."""
+    m, k = 700, 4000
+    ws = C.Workspace(m, k, n)
+    dense = _weights(m, k, 0.3, 5)
+    w = _csr(C, dense, ws)
+    x = torch.randn(k, n, device="cuda", generator=_gen(n))
+    b, e = (int(v) for v in w.row_ptr[[37, 38]])
+    if how == "twice":
+        w.col_idx[b + 9] = w.col_idx[b + 8]
+    else:
+        perm = torch.arange(e - b - 1, -1, -1) if how == "reversed" else torch.randperm(e - b)
+        w.col_idx[b:e] = w.col_idx[b:e][perm.cuda()]
+        w.val[b:e] = w.val[b:e][perm.cuda()]
+    full = torch.zeros(m, k, device="cuda", dtype=torch.float64)
+    nnz = int(w.row_ptr[-1])
+    rows = torch.repeat_interleave(torch.arange(m, device="cuda"), (w.row_ptr[1:] - w.row_ptr[:-1]).long())
+    full.index_put_((rows, w.col_idx[:nnz].long()), w.val[:nnz].double(), accumulate=True)
+    mag = torch.zeros_like(full).index_put_((rows, w.col_idx[:nnz].long()), w.val[:nnz].double().abs(),
+                                            accumulate=True)
+    y = torch.full((m, n), float("nan"), device="cuda")
+    C.spmm_fwd(w, x, y, ws)
+    lens = (w.row_ptr[1:] - w.row_ptr[:-1]).double()[:, None]
+    assert bool(((y.double() - full @ x.double()).abs() <= (lens + 2) * U * (mag @ x.double().abs())).all())
+    assert ws.status()[0] == 0
