@@ -38,10 +38,9 @@
 // the same tensor and shared memory), 10 for the partial sums (20 MB written
 // and read in L2).
 //
-// Values a factor can't take here (2^50 and more, infinities, NaN) turn the
-// scale of their row or chunk into NaN, which ends as a NaN in the sums they
-// touch; such entries of Y are computed again from the CSR row. Rows out of
-// order or with an entry twice make the whole product run by gathering.
+// Operands that the tensor cores can't take (values of 2^50 and more, infinities,
+// NaN, rows out of order or with an entry twice) are marked by the first kernel
+// and make the whole product run by gathering (st_gather).
 #include "spmm_tc.cuh"
 #include "tc_pair.cuh"
 
@@ -96,14 +95,6 @@ __device__ __forceinline__ void mma_f16_pair_down11(uint32_t tmem_d, uint64_t ad
         " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p, 11;\n}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc)
         : "memory");
-}
-
-// Entry (row, c) of the product from the CSR row, as the sparse kernel adds it.
-static __device__ __noinline__ float st_entry(const StArgs &a, int64_t row, int64_t c) {
-    float sum = 0.f;
-    for (int32_t k = a.row_ptr[row]; k < a.row_ptr[row + 1]; ++k)
-        sum = fmaf(__ldg(a.val + k), __ldg(a.x + (int64_t)__ldg(a.col + k) * a.n + c), sum);
-    return sum;
 }
 
 __device__ __forceinline__ float st_finish(const StArgs &a, int64_t row, int64_t c, float v) {
@@ -188,11 +179,6 @@ __device__ __forceinline__ void st_write(const StArgs &a, int tile, uint32_t ran
     float v[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = sum[i] * wsc;
-    if (isnan(v[0])) {
-        for (int i = 0; i < 8 && col + i < a.n; ++i)
-            a.y[row * a.n + col + i] = st_finish(a, row, col + i, st_entry(a, row, col + i));
-        return;
-    }
     if (a.bias || a.relu || a.mask) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -548,7 +534,7 @@ static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int64_t capacity, int
     return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)4 * n * st_ld(k)) +
            st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) + st_align((size_t)4 * rows) +
            st_align((size_t)4 * chunks * ceil_div(n, n_tile / 4)) +
-           st_align((size_t)ceil_div(rows, kTcGroup)) +
+           st_align((size_t)ceil_div(rows, kTcGroup) + chunks * ceil_div(n, n_tile / 4)) +
            st_align((size_t)8 * ceil_div(rows, 256) * ceil_div(n, n_tile)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
 }
 constexpr int32_t kStMinRows = 256, kStMinK = 1024, kStMinN = 65;
@@ -621,7 +607,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)));
     plan->prep.wscale = reinterpret_cast<float *>(take((size_t)4 * rows));
     plan->prep.xscale = reinterpret_cast<float *>(take((size_t)4 * chunks * ceil_div(n, n_tile / 4)));
-    plan->prep.num_marks = ceil_div(rows, kTcGroup);
+    plan->prep.num_marks = ceil_div(rows, kTcGroup) + chunks * ceil_div(n, n_tile / 4);
     plan->prep.marks = reinterpret_cast<uint8_t *>(take((size_t)plan->prep.num_marks));
     plan->prep.counters = 2 * plan->tiles;
     plan->prep.cnt = reinterpret_cast<uint32_t *>(take((size_t)4 * plan->prep.counters));

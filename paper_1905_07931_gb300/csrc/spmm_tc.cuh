@@ -24,12 +24,12 @@ struct SpmmTcPrep {
     uint32_t *parts;     // [capacity] high (bits 0-15) and low part of each entry, rows scaled by a power of two,
     uint16_t *place;     // and its byte offset in its group's 16 x 128 byte block of the GEMM's operand
     int32_t *start;      // [groups][chunks + 1] first entry of each group's chunk
-    float *wscale;       // [rows] undoes the rows' scale (NaN: the row holds a value the path cannot take)
+    float *wscale;       // [rows] undoes the rows' scale
     __half *xp;          // [2][n][ld] high and low parts of X transposed, scaled per chunk and `width` columns
-    float *xscale;       // [chunks][ceil(n / width)] undoes that (NaN likewise)
+    float *xscale;       // [chunks][ceil(n / width)] undoes that
     int32_t k, ld, chunks, width;
     int32_t vec;         // rows of X may be read as float4
-    uint8_t *marks;      // [groups] 1: the group holds rows that the tensor cores can't take
+    uint8_t *marks;      // [groups], then [chunks][ceil(n / width)] of X: 1: rows or values that the tensor cores can't take
     int32_t num_marks;
     uint32_t *cnt;       // [counters] of the tensor-core kernel's cut tiles, zeroed here: a kernel that gave up
     int32_t counters;    // waiting leaves nothing behind for the next call
@@ -56,7 +56,9 @@ int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t
                    cudaStream_t s);
 
 // Values a factor may take on the tensor-core path (products and sums of
-// these stay far inside float32's range).
+// these stay far inside float32's range). With larger ones, infinities or NaN
+// the whole product is gathered instead: it then costs about what the sparse
+// kernel would.
 constexpr uint32_t kTcLimitBits = (127u + 50u) << 23;   // 2^50
 
 // The power of two that brings a value of magnitude bits `mx` into [2^14,
@@ -80,10 +82,10 @@ __device__ __forceinline__ uint32_t tc_place(int r, int j) {
 }
 
 // X's planes of one chunk (64 features) and `width` columns (64 or 32), which
-// share a scale: a block of 256 threads, a lane holds the features j and j +
+// share a scale (marks_w: the marks of W before X's): a block of 256 threads, a lane holds the features j and j +
 // 32 of its warp's eighth of the columns, read once. s_max: 8 words.
 __device__ __forceinline__ void spmm_tc_prep_x(const SpmmTcPrep &a, const float *__restrict__ x, int32_t n, int chunk,
-                                               int block, uint32_t *s_max) {
+                                               int block, int marks_w, uint32_t *s_max) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = a.width / 8;
     const int c0 = block * a.width + warp * per;
@@ -116,8 +118,12 @@ __device__ __forceinline__ void spmm_tc_prep_x(const SpmmTcPrep &a, const float 
     const bool bad = mx >= kTcLimitBits;   // infinities and NaN too
     float down, up;
     fp16_scales(mx, down, up);
-    if (threadIdx.x == 0)
-        a.xscale[chunk * ((n + a.width - 1) / a.width) + block] = bad ? __uint_as_float(0x7fc00000u) : up;
+    if (threadIdx.x == 0) {
+        const int at = chunk * ((n + a.width - 1) / a.width) + block;
+        a.marks[marks_w + at] = bad;
+        a.xscale[at] = up;
+    }
+    if (bad) return;
     const int64_t plane = (int64_t)n * a.ld;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -127,7 +133,7 @@ __device__ __forceinline__ void spmm_tc_prep_x(const SpmmTcPrep &a, const float 
             const int j = chunk * kTcChunk + h * 32 + lane;
             if (j >= a.k) continue;
             __half hi, lo;
-            fp16_split(bad ? 0.f : v[h][e] * down, hi, lo);
+            fp16_split(v[h][e] * down, hi, lo);
             __half *p = a.xp + (int64_t)(c0 + e) * a.ld + j;
             p[0] = hi;
             p[plane] = lo;
@@ -208,11 +214,10 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
     for (int q = 0; q < 2; ++q) {
         const int32_t r = group * kTcGroup + warp * 2 + q;
         const uint32_t m = __reduce_max_sync(0xffffffffu, mx[q]);
-        const bool bad = m >= kTcLimitBits;
+        unfit |= m >= kTcLimitBits;   // (infinities and NaN too)
         float up;
         fp16_scales(m, down[q], up);
-        if (bad) down[q] = 0.f;   // (an infinity becomes NaN; its row's sums are NaN in any case)
-        if (lane == 0 && r < rows) a.wscale[r] = bad ? __uint_as_float(0x7fc00000u) : up;
+        if (lane == 0 && r < rows) a.wscale[r] = up;
     }
     __shared__ int32_t s_sum[9];
     const int32_t base = __ldg(row_ptr + group * kTcGroup);
@@ -297,9 +302,9 @@ __device__ __forceinline__ void spmm_tc_prep(const SpmmTcPrep &a, const int32_t 
     const int busy = ws % grid, idle = grid - busy;
     if (busy && idle >= grid / 4) {
         if (b < busy) return;
-        for (int i = b - busy; i < xs; i += idle) spmm_tc_prep_x(a, x, n, i / nb, i % nb, s_max);
+        for (int i = b - busy; i < xs; i += idle) spmm_tc_prep_x(a, x, n, i / nb, i % nb, ws, s_max);
     } else {
-        for (int i = b; i < xs; i += grid) spmm_tc_prep_x(a, x, n, i / nb, i % nb, s_max);
+        for (int i = b; i < xs; i += grid) spmm_tc_prep_x(a, x, n, i / nb, i % nb, ws, s_max);
     }
 }
 
