@@ -198,6 +198,11 @@ __device__ __forceinline__ void st_write(const StArgs &a, int tile, uint32_t ran
 // shares whose pairs gave up waiting (from bit 8). The first kernel of every
 // product zeroes the counters.
 constexpr uint32_t kStPartsMask = 0xff;
+// How long a pair waits for the others' parts: 15 us at 2 GHz, or this many
+// looks (each a round trip to L2, up to 1 to 2 us under the load of the
+// partial sums: by their number alone the wait could last 25 times as long).
+constexpr long long kStShareClocks = 30000;
+constexpr int kStSharePolls = 400;
 
 // One pair's part in adding up a cut tile; `seen` is what its counter was when
 // it counted in.
@@ -217,10 +222,11 @@ __device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, 
             __threadfence();
         } else if (todo) {
             bool all = false;
-            for (int i = 0; i < 400; ++i) {
+            const long long begun = clock64();
+            for (int i = 0; i < kStSharePolls; ++i) {
                 uint32_t now;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(cnt) : "memory");
-                if ((all = (int)(now & kStPartsMask) == parts)) break;
+                if ((all = (int)(now & kStPartsMask) == parts) || clock64() - begun > kStShareClocks) break;
                 __nanosleep(20);
             }
             // gives up; whoever counts in last takes the share, unless it just has
@@ -501,8 +507,8 @@ __global__ void __launch_bounds__(kStThreads, 1)
         }
         // The cut tiles: their pairs share the work of adding the partial
         // sums (in pair order, so the result does not depend on who adds).
-        // All pairs finish at about the same time: each waits a moment (some
-        // 15 us at most) until a tile's parts are all there and takes its own
+        // All pairs finish at about the same time: each waits a moment
+        // (kStShareClocks) until a tile's parts are all there and takes its own
         // share of the columns. One that has waited in vain leaves a note and
         // goes; the last pair to count in does the shares of those, so
         // nothing depends on all pairs being resident at once.

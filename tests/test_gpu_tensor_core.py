@@ -171,3 +171,25 @@ def test_product_with_values_out_of_range_costs_a_sparse_product(C):
             y[hit], ref[hit] = 0, 0
         assert bool(((y.double() - ref).abs() <= (lens + 3) * U * mag).all()), what
     assert ws.status()[0] == 0
+
+
+def test_product_beside_another_kernel(C):
+    """While another stream's kernel holds most of the GPU the pairs of shared tiles are not resident together: each
+    gives up its wait, whoever counts in last does its share, and the sums are the same."""
+    m, k, n = 4096, 4096, 256
+    ws = C.Workspace(m, k, n)
+    w = _csr(C, _weights(m, k, 0.2, 8), ws)
+    x = torch.randn(k, n, device="cuda", generator=_gen(9))
+    want, got = torch.empty(m, n, device="cuda"), torch.empty(m, n, device="cuda")
+    C.spmm_fwd(w, x, want, ws)
+    side, blocks = torch.cuda.Stream(), 120
+    out = torch.empty(blocks * 512, device="cuda")
+    torch.cuda.synchronize()
+    for iters in (1 << 15, 1 << 17):
+        assert C.lib().csrt_fma_peak_run(out.data_ptr(), blocks, iters, None, side.cuda_stream) == 0
+        for _ in range(5):
+            got.fill_(float("nan"))
+            C.spmm_fwd(w, x, got, ws)
+            assert torch.equal(_bits(got), _bits(want))
+        side.synchronize()
+    assert ws.status()[0] == 0
