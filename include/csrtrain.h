@@ -188,11 +188,17 @@ int csr_transpose(csrt_csr *w, void *ws, size_t ws_bytes, void *stream);
 /* spmm_fwd -- Section 3.2.1 (dense x compressed', the forward pass).
  * Y[M x n] = W X[K x n]: Y[i, c] = sum over stored k of row i of
  * val[k] * X[col_idx[k], c], float32 accumulation. Y is overwritten.
- * Matrices dense enough that multiplying the zeros is cheaper (from about 5%
- * of at least 1024 columns, n > 64) run on the tensor cores: both factors in
- * two fp16 parts each (22 to 23 bits), float32 sums, an error below that of
- * the float32 chains it replaces; the same call on the same data always gives
- * the same bits. Needs the workspace of csrt_workspace_bytes.
+ * Matrices dense enough that multiplying the zeros is cheaper (at least 256
+ * rows of 1024 columns, n > 64, from 4% to 9% of the entries on, by shape; not
+ * where that would take more) run on the tensor cores: both factors as three
+ * bf16 parts each, all 24 bits, float32 sums. An element's error is that of
+ * its own terms, whatever the magnitudes around it: for sums of some hundred
+ * terms below that of the float32 chains it replaces, for a sum of one term one
+ * rounding and at most 2^-24 of it. Values of 2^28 and more, infinities, NaN,
+ * and rows out of order are handled as the sparse kernels do, at their price.
+ * The same call on the same data always gives the same bits, but those of the
+ * sparse kernels differ: a workspace smaller than csrt_workspace_bytes is
+ * accepted as long as it holds what those need, and then they run.
  * Products with n <= 16 (64 for float4-aligned X and Y) stream col_idx and
  * val through shared memory with bulk copies when both arrays are 16-byte
  * aligned (else a 32-lane kernel runs); a copy that does not complete within

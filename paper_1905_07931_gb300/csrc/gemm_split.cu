@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(kGsThreads, 1)
                         for (int q = 0; q < 6; ++q)
 #pragma unroll
                             for (int k = 0; k < kGsChunk / 16; ++k)
-                                mma_f16_pair(d, smem_desc_sw128(st + pa[q] * kGsSlice + hf * 64 + k * 32),
-                                             smem_desc_sw128(st + (3 + pb[q]) * kGsSlice + hf * 64 + k * 32), kGsIdesc,
+                                mma_f16_pair(d, smem_desc_lo(st + pa[q] * kGsSlice + hf * 64 + k * 32),
+                                             smem_desc_lo(st + (3 + pb[q]) * kGsSlice + hf * 64 + k * 32), kGsIdesc,
                                              (q > 0 || k > 0) ? 1u : 0u);
                         if (hf == halves - 1) mma_commit_pair(empty + s);
                         mma_commit_pair(accf + b);

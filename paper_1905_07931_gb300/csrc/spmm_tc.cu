@@ -2,23 +2,21 @@
 // enough that gathering a row of X per stored entry (n floats from L2 each)
 // costs more than multiplying the zeros.
 //
-// The product runs as a GEMM over all of W's columns in float32 accuracy.
-// Every factor is split into two fp16 parts, v = 2^s (hi + 2^-11 lo), with s
-// such that the largest magnitude that shares it lies in [2^14, 2^15): one s
-// per row of W, one per 64 features (rows) and 64 columns of X. hi and lo hold
-// 22 to 23 bits of every value down to 2^-29 of that largest one. Three products are taken,
-// hi lo' + lo hi' first and then hi hi' on top of them (the accumulator's
-// scale-input-d brings the first two down by 2^-11); lo lo' is below 2^-22.
-// tcgen05.mma truncates when it adds into its accumulator, so the sum of each
-// 64-column chunk of the reduction (four steps of hi hi') is read back and
-// added to float32 register sums, scaled by the chunk's power of two, with
-// round to nearest. Measured error against 64 bits: 1.2e-7 to 1.7e-7 where
-// the float32 chain of the sparse kernel has 1.6e-7 to 5.5e-7 (rows of 150 to
-// 2000 entries); layers whose rows hold fewer than 160 entries on average
-// keep the sparse kernel, whose short chains are more exact.
+// The product runs as a GEMM over all of W's columns in float32 accuracy: both
+// factors as sums of three bf16 parts, all 24 bits of every value and all of
+// float32's exponents below 2^28, six of the nine products of parts, x1 w1 in
+// sums of 64 columns that are added up with round to nearest (split_bf16.cuh).
+// An element of Y thus has no part in the magnitudes of its neighbours: two
+// fp16 parts, with a power of two per row of W and per 64 features x 64 columns
+// of X, took half the products, but a sample 1e-16 times as large as another of
+// its block was lost (relative error 0.2), W times unit vectors did not return
+// W, and a sum of one term had up to 5.1e-7 where float32's rounding is 6e-8.
+// Measured error against 64 bits: 0.7e-7 to 1.6e-7 where the float32 chain of the
+// sparse kernel has 1.7e-7 to 7.8e-7 (rows of 120 to 2000 entries); layers whose
+// rows hold fewer than 160 entries on average keep the sparse kernel.
 //
 // W never exists densely in memory: the first kernel (spmm_tc.cuh) sorts its
-// split entries by groups of 16 rows and chunks of 64 columns, and eight warps
+// entries by groups of 16 rows and chunks of 64 columns, and eight warps
 // of each CTA put a chunk's entries into the cleared shared-memory operand of
 // the MMA (6 bytes per entry instead of 4 per element: written out as dense
 // planes, a layer at 5% took 52 us instead of 48, at 50% 83 instead of 96).
@@ -29,16 +27,10 @@
 // add the parts up in pair order (st_share). Where there are enough tiles for
 // the GPU no tile is cut.
 //
-// Measured (GB300; the sparse kernel's time in brackets), rows x inner x n:
-// 4096 x 4096 x 256 at 20% 61 us (160), at 50% 96 (385), x 1024 at 5% 107
-// (170), at 50% 177 (1520), x 255 at 5% 51 (125); 4096 x 9216 x 256 at 5% 79
-// (99). At 4096 x 4096 x 256 and 5%: 10 us for the first kernel, 3 until the
-// first chunk's MMAs, 1.25 to 1.4 us per chunk (14 per pair; the MMAs alone
-// 1.0, slowed by the reading back and the expanding warps' stores, which use
-// the same tensor and shared memory), 10 for the partial sums (20 MB written
-// and read in L2).
+// The MMAs take 1.7 us per chunk (six products; 24 of K = 16), with the
+// operands and the reading back 1.9.
 //
-// Operands that the tensor cores can't take (values of 2^50 and more, infinities,
+// Operands that the tensor cores can't take (values of 2^28 and more, infinities,
 // NaN, rows out of order or with an entry twice) are marked by the first kernel
 // and make the whole product run by gathering (st_gather).
 #include "spmm_tc.cuh"
@@ -47,6 +39,7 @@
 namespace csrt {
 
 constexpr int kStChunk = kTcChunk;
+static_assert(kStChunk == kSplitChunk, "a stage is a sum of x1 w1");
 // Warps: 0 TMA, 1 MMA (2 and 3 idle), eight that expand W (a group of 16 rows
 // each), sixteen that add up and write. kStSplitRegs: what their shares come to
 // (the launch is found to hold them before it is used; ptxas gives 896 x 72).
@@ -58,8 +51,8 @@ constexpr int kStSplitRegs =
 static_assert(kStSplitRegs <= kStThreads * 72, "register split");
 constexpr int kStASlice = 128 * kStChunk * 2;
 template <int kN> __host__ __device__ constexpr int st_bslice() { return kN / 2 * kStChunk * 2; }
-template <int kN> __host__ __device__ constexpr int st_stage() { return 2 * (kStASlice + st_bslice<kN>()); }
-template <int kN> __host__ __device__ constexpr int st_stages() { return kN == 256 ? 3 : 4; }
+template <int kN> __host__ __device__ constexpr int st_stage() { return 3 * (kStASlice + st_bslice<kN>()); }
+template <int kN> __host__ __device__ constexpr int st_stages() { return kN == 256 ? 2 : 3; }
 template <int kN> __host__ __device__ constexpr int st_smem() { return st_stages<kN>() * st_stage<kN>() + 256 + 1024; }
 static_assert(st_smem<256>() <= 232448 && st_smem<128>() <= 232448, "shared memory per block");
 
@@ -67,10 +60,10 @@ struct StArgs {
     const int32_t *row_ptr, *col;
     const float *val;
     int32_t rows, k, n;
-    const uint32_t *parts;
+    const float *sorted;
     const uint16_t *place;
     const int32_t *start;
-    const float *x, *wscale, *xscale;
+    const float *x;
     float *y, *partial;
     uint32_t *cnt;
     const uint8_t *marks;
@@ -88,13 +81,6 @@ __device__ __forceinline__ int32_t ld_row_end(const int32_t *p) {
     int32_t v;
     asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-__device__ __forceinline__ void mma_f16_pair_down11(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n"
-        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p, 11;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc)
-        : "memory");
 }
 
 __device__ __forceinline__ float st_finish(const StArgs &a, int64_t row, int64_t c, float v) {
@@ -164,21 +150,17 @@ __device__ __forceinline__ float *st_slot(const StArgs &a, int pair, bool beginn
     return a.partial + ((int64_t)(pair * 2 + (beginning ? 1 : 0)) * 2 + rank) * 128 * kN;
 }
 
-__device__ __forceinline__ float st_row_scale(const StArgs &a, int tile, uint32_t rank, int q) {
-    const int64_t row = (int64_t)(tile / a.tiles_n) * 256 + rank * 128 + q * 32 + (threadIdx.x & 31);
-    return row < a.rows ? __ldg(a.wscale + row) : 0.f;
-}
 // Eight columns (c .. c + 7 of the tile) of row 32q + lane of the CTA's half
-// of a tile: W's row scale, the epilogue, Y.
+// of a tile: the sums without the factors' scales, the epilogue, Y.
 template <int kN>
-__device__ __forceinline__ void st_write(const StArgs &a, int tile, uint32_t rank, int q, int c, const float *sum,
-                                         float wsc) {
+__device__ __forceinline__ void st_write(const StArgs &a, int tile, uint32_t rank, int q, int c,
+                                         const float *sum) {
     const int64_t row = (int64_t)(tile / a.tiles_n) * 256 + rank * 128 + q * 32 + (threadIdx.x & 31);
     const int64_t col = (int64_t)(tile % a.tiles_n) * kN + c;
     if (row >= a.rows || col >= a.n) return;
     float v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = sum[i] * wsc;
+    for (int i = 0; i < 8; ++i) v[i] = sum[i] * kSplitDown;
     if (a.bias || a.relu || a.mask) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -238,7 +220,6 @@ __device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, 
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kStEpiWarps) : "memory");
     uint32_t todo = *state;
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kStEpiWarps) : "memory");   // state is read
-    const float wsc = st_row_scale(a, tile, rank, q);
     for (; todo; todo &= todo - 1) {
         const int s = __ffs((int)todo) - 1;
         for (int c = kUnits * s / shares; c < kUnits * (s + 1) / shares; ++c) {
@@ -258,7 +239,7 @@ __device__ __noinline__ void st_share(const StArgs &a, int64_t units, int pair, 
                         for (int i = 0; i < 8; ++i) v[i] += x[o][i];
                     }
             }
-            st_write<kN>(a, tile, rank, q, h * (kN / 4) + c * 8, v, wsc);
+            st_write<kN>(a, tile, rank, q, h * (kN / 4) + c * 8, v);
         }
     }
 }
@@ -274,13 +255,13 @@ __global__ void __launch_bounds__(kStThreads, 1)
     }
     constexpr int kStages = st_stages<kN>(), kStage = st_stage<kN>(), kBSlice = st_bslice<kN>();
     constexpr int kCols = kN / 4;   // columns of an epilogue warp
-    constexpr uint32_t kIdesc = idesc_f16(0, 256, kN);
+    constexpr uint32_t kIdesc = idesc_f16(1, 256, kN);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStage);
     uint64_t *empty = full + kStages;
-    uint64_t *accf = empty + kStages;
-    uint64_t *acce = accf + 2;
+    uint64_t *accf = empty + kStages;   // [2] the accumulator of x1 w1, that of the small products: ready
+    uint64_t *acce = accf + 2;          // [2] read (the leader's: all warps of both CTAs)
     uint64_t *fin = acce + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
     __shared__ volatile int s_abort;
@@ -328,48 +309,69 @@ __global__ void __launch_bounds__(kStThreads, 1)
         else st_gather<1>(a);
     } else if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kStProdRegs));
+        // (few registers here: what changes is the stage, its barriers' parity, and
+        // those of the accumulators)
+        const int stages = (int)(u_end - u_begin);
+        int ch = (int)(u_begin % a.chunks), st = 0;
+        uint32_t turn = 0;   // bit 0: parity of the stages' round; 1, 2: of the accumulators
         if (warp == 0 && lane == 0) {
-            int it = 0;
-            int tile = (int)(u_begin / a.chunks), ch = (int)(u_begin % a.chunks);
-            for (int64_t u = u_begin; u < u_end && !s_abort; ++u, ++it) {
-                const int c0 = (tile % a.tiles_n) * kN + (int)rank * (kN / 2);
-                const int s = it % kStages;
-                if (!mbar_wait_or_abort(empty + s, ((it / kStages) & 1) ^ 1, &s_abort)) break;
-                if (rank == 0) mbar_expect_tx(full + s, 4 * kBSlice);
-                const uint32_t bar = map_to_rank(full + s, 0);
-                uint8_t *st = smem + s * kStage + 2 * kStASlice;
-                tma_load_2d_pair(st, &map_x, ch * kStChunk, c0, bar);
-                tma_load_2d_pair(st + kBSlice, &map_x, ch * kStChunk, a.n + c0, bar);
+            int c0 = (int)(u_begin / a.chunks % a.tiles_n) * kN + (int)rank * (kN / 2);
+            int done = 0;
+            for (; done < stages && !s_abort; ++done) {
+                if (!pair_wait(empty + st, (turn & 1) ^ 1, &s_abort)) break;
+                if (rank == 0) mbar_expect_tx(full + st, 6 * kBSlice);
+                const uint32_t bar = map_to_rank(full + st, 0);
+                uint8_t *to = smem + st * kStage + 3 * kStASlice;
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+                    tma_load_2d_pair(to + p * kBSlice, &map_x, ch * kStChunk, p * a.n + c0, bar);
                 if (++ch == a.chunks) {
                     ch = 0;
-                    ++tile;
+                    c0 += kN;
+                    if (c0 >= a.tiles_n * kN) c0 = (int)rank * (kN / 2);
                 }
+                if (++st == kStages) st = 0, turn ^= 1;
             }
             // every load of both CTAs must land before the pair may exit
             if (rank == 0)
-                for (int i = imax(0, it - kStages); i < it; ++i) mbar_wait(full + i % kStages, (i / kStages) & 1);
+                for (int i = imax(0, done - kStages); i < done; ++i) mbar_wait(full + i % kStages, (i / kStages) & 1);
         } else if (warp == 1 && lane == 0 && rank == 0) {
-            int it = 0;
-            for (int64_t u = u_begin; u < u_end && !s_abort; ++u, ++it) {
-                const int s = it % kStages, b = it & 1;
-                if (!mbar_wait_or_abort(acce + b, ((it >> 1) & 1) ^ 1, &s_abort)) break;
-                if (!mbar_wait_or_abort(full + s, (it / kStages) & 1, &s_abort)) break;
+            int in_flush = 0;
+            for (int done = 1; done <= stages && !s_abort; ++done) {
+                if (!pair_wait(full + st, turn & 1, &s_abort)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint8_t *ah = smem + s * kStage, *al = ah + kStASlice;
-                const uint8_t *bh = ah + 2 * kStASlice, *bl = bh + kBSlice;
-                const uint32_t d = tmem + (uint32_t)(b * kN);
+                // (a descriptor's low bits are the address in units of 16 bytes)
+                const uint32_t da = smem_desc_lo(smem + st * kStage);
+                if (in_flush == 0) {
+                    if (!pair_wait(acce + 1, (turn >> 2) ^ 1, &s_abort)) break;
+                    turn ^= 4;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
+                // the small products first (while they run, the sum of x1 w1 before
+                // is read): parts of W and of X by steps of four bits
+#pragma unroll 1
+                for (int q = 0; q < 20; q += 4) {
+                    const uint32_t qa = da + (kSplitPartsA >> q & 3) * (kStASlice >> 4);
+                    const uint32_t qb = da + (3 * kStASlice >> 4) + (kSplitPartsB >> q & 3) * (kBSlice >> 4);
+#pragma unroll
+                    for (int k = 0; k < kStChunk / 16; ++k)
+                        mma_f16_pair(tmem + kN, qa + k * 2, qb + k * 2, kIdesc, k > 0 ? 1 : in_flush | q);
+                }
+                if (!pair_wait(acce, (turn >> 1 & 1) ^ 1, &s_abort)) break;
+                turn ^= 2;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                 for (int k = 0; k < kStChunk / 16; ++k)
-                    mma_f16_pair(d, smem_desc_sw128(ah + k * 32), smem_desc_sw128(bl + k * 32), kIdesc, k > 0);
-#pragma unroll
-                for (int k = 0; k < kStChunk / 16; ++k)
-                    mma_f16_pair(d, smem_desc_sw128(al + k * 32), smem_desc_sw128(bh + k * 32), kIdesc, 1u);
-                mma_f16_pair_down11(d, smem_desc_sw128(ah), smem_desc_sw128(bh), kIdesc);
-#pragma unroll
-                for (int k = 1; k < kStChunk / 16; ++k)
-                    mma_f16_pair(d, smem_desc_sw128(ah + k * 32), smem_desc_sw128(bh + k * 32), kIdesc, 1u);
-                mma_commit_pair(empty + s);
-                mma_commit_pair(accf + b);
+                    mma_f16_pair(tmem, da + k * 2, da + (3 * kStASlice >> 4) + k * 2, kIdesc, k > 0);
+                mma_commit_pair(accf);
+                ++in_flush;
+                mma_commit_pair(empty + st);
+                if (++ch == a.chunks) ch = 0;
+                if (in_flush == kSplitFlush || ch == 0 || done == stages) {
+                    mma_commit_pair(accf + 1);
+                    in_flush = 0;
+                }
+                if (++st == kStages) st = 0, turn ^= 1;
             }
             asm volatile(
                 "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(fin))
@@ -379,7 +381,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
     } else if (warp < 4 + kStExpandWarps) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kStExpandRegs));
         // An expanding warp: one group of 16 rows. Per chunk it clears their
-        // 128 bytes in both planes and puts the entries' parts at their
+        // 128 bytes in the three planes and puts the entries' parts at their
         // places, 256 entries at a time. The next entries are asked for as
         // soon as these are in place: their latency (1000 clocks under load)
         // passes while the MMAs of the stages ahead run. The bounds of 31
@@ -394,12 +396,13 @@ __global__ void __launch_bounds__(kStThreads, 1)
             ch_ends = ch;
             ends = g < groups ? __ldg(a.start + (int64_t)g * (a.chunks + 1) + imin(ch + lane, a.chunks)) : 0;
         };
-        uint32_t part[8], place[8];
+        float val[8];
+        uint32_t place[8];
         auto fetch = [&](int32_t i, int32_t hi) {
 #pragma unroll
             for (int h = 0; h < 8; ++h) {
                 const bool on = i + h * 32 + lane < hi;
-                part[h] = on ? __ldg(a.parts + i + h * 32 + lane) : 0u;
+                val[h] = on ? __ldg(a.sorted + i + h * 32 + lane) : 0.f;
                 place[h] = on ? __ldg(a.place + i + h * 32 + lane) : 0xffffu;
             }
         };
@@ -422,30 +425,37 @@ __global__ void __launch_bounds__(kStThreads, 1)
             }
             const int s = it % kStages;
             uint8_t *base = smem + s * kStage + e * (kTcGroup * 128);
-            if (!__all_sync(0xffffffffu, mbar_wait_or_abort(empty + s, ((it / kStages) & 1) ^ 1, &s_abort))) break;
+            if (!__all_sync(0xffffffffu, pair_wait(empty + s, ((it / kStages) & 1) ^ 1, &s_abort))) break;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                *reinterpret_cast<uint4 *>(base + i * 512 + lane * 16) = make_uint4(0, 0, 0, 0);
-                *reinterpret_cast<uint4 *>(base + kStASlice + i * 512 + lane * 16) = make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+                    *reinterpret_cast<uint4 *>(base + p * kStASlice + i * 512 + lane * 16) = make_uint4(0, 0, 0, 0);
             }
             __syncwarp();
             while (true) {
 #pragma unroll
-                for (int h = 0; h < 8; ++h)
-                    if (place[h] != 0xffffu) {
-                        *reinterpret_cast<uint16_t *>(base + place[h]) = (uint16_t)part[h];
-                        *reinterpret_cast<uint16_t *>(base + kStASlice + place[h]) = (uint16_t)(part[h] >> 16);
+                for (int h = 0; h < 8; h += 2) {
+                    __nv_bfloat162 part[3];
+                    split_bf16(make_float2(val[h], val[h + 1]), part[0], part[1], part[2]);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        uint8_t *at = base + p * kStASlice;
+                        if (place[h] != 0xffffu) *reinterpret_cast<__nv_bfloat16 *>(at + place[h]) = part[p].x;
+                        if (place[h + 1] != 0xffffu) *reinterpret_cast<__nv_bfloat16 *>(at + place[h + 1]) = part[p].y;
                     }
+                }
                 lo += 256;
                 if (lo >= hi) break;
                 fetch(lo, hi);
             }
-            fetch(lo_n, hi_n);
-            lo = lo_n;
-            hi = hi_n;
+            // (loads in flight would hold up the fence: the next chunk's come after it)
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(map_to_rank(full + s, 0));
+            fetch(lo_n, hi_n);
+            lo = lo_n;
+            hi = hi_n;
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kStEpiRegs));
@@ -453,7 +463,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
         const int h = (warp - 4 - kStExpandWarps) >> 2;   // column quarter of the tile
         const int tid = threadIdx.x - 32 * (4 + kStExpandWarps);
         const uint32_t acce0 = map_to_rank(acce, 0), acce1 = map_to_rank(acce + 1, 0);
-        int it = 0, tile_e = -1, tile_b = -1;
+        int sums = 0, flushes = 0, tile_e = -1, tile_b = -1;
         uint32_t seen_e = 0, seen_b = 0;   // (thread 0)
         bool ok = true;
         for (int64_t u = u_begin; u < u_end;) {
@@ -462,31 +472,32 @@ __global__ void __launch_bounds__(kStThreads, 1)
             float acc[kCols];
 #pragma unroll
             for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
-            const int nb = (a.n + kCols - 1) / kCols, xb = imin((tile % a.tiles_n) * 4 + h, nb - 1);
-            float sc = __ldg(a.xscale + ch0 * nb + xb);
-            for (int ch = ch0; ch < ch1; ++ch, ++it) {
-                const int b = it & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait_or_abort(accf + b, (it >> 1) & 1, &s_abort));
-                if (!ok) break;
+            // (b = 0: the accumulator of x1 w1; 1: that of the small products)
+            auto add_up = [&](int b, int times) {
+                ok = __all_sync(0xffffffffu, pair_wait(accf + b, times & 1, &s_abort));
+                if (!ok) return;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                 for (int c = 0; c < kCols; c += 16) {
                     uint32_t r[16];
                     tmem_ld_16cols(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kN + h * kCols + c), r);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[c + i] = fmaf(__uint_as_float(r[i]), sc, acc[c + i]);
+                    for (int i = 0; i < 16; ++i) acc[c + i] += __uint_as_float(r[i]);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(b ? acce1 : acce0);
-                sc = __ldg(a.xscale + imin(ch + 1, a.chunks - 1) * nb + xb);
+            };
+            const int sums_here = ch1 - ch0;
+            for (int i = 1; i <= sums_here && ok; ++i) {
+                add_up(0, sums++);
+                if (ok && (i % kSplitFlush == 0 || i == sums_here)) add_up(1, flushes++);
             }
             if (!ok) break;
             u += ch1 - ch0;
             if (ch0 == 0 && ch1 == a.chunks) {
-                const float wsc = st_row_scale(a, tile, rank, q);
 #pragma unroll
-                for (int c = 0; c < kCols; c += 8) st_write<kN>(a, tile, rank, q, h * kCols + c, acc + c, wsc);
+                for (int c = 0; c < kCols; c += 8) st_write<kN>(a, tile, rank, q, h * kCols + c, acc + c);
                 continue;
             }
             // A partial sum: left in the workspace, counted in. (A pair's
@@ -537,9 +548,8 @@ static int st_max_pairs() { return imax(1, num_sms() / 2); }
 // `capacity` entries and n columns.
 static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int64_t capacity, int n_tile) {
     const int64_t chunks = ceil_div(k, kStChunk);
-    return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)4 * n * st_ld(k)) +
-           st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) + st_align((size_t)4 * rows) +
-           st_align((size_t)4 * chunks * ceil_div(n, n_tile / 4)) +
+    return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)6 * n * st_ld(k)) +
+           st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) +
            st_align((size_t)ceil_div(rows, kTcGroup) + chunks * ceil_div(n, n_tile / 4)) +
            st_align((size_t)8 * ceil_div(rows, 256) * ceil_div(n, n_tile)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
 }
@@ -575,7 +585,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     // (microseconds; the partial sums take 4 us and 2.2 us for each eighth of
     // a tile's columns that a pair has to add up).
     const int max_pairs = st_max_pairs();
-    const double t_unit = n_tile == 256 ? 1.25 : 0.85;
+    const double t_unit = n_tile == 256 ? 1.95 : 1.75;
     const int cut_pairs = (int)imin<int64_t>(units, max_pairs);
     const double whole = (double)ceil_div(plan->tiles, max_pairs) * chunks * t_unit;
     const double cut = (double)ceil_div<int64_t>(units, cut_pairs) * t_unit + 4.0 +
@@ -585,17 +595,18 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     // The number of entries from which this path is the faster one: both
     // times are fits to measurements over 512..9216 rows and columns, 1% to
     // 50% and 100 to 1024 columns of X (within 15%):
-    //   here    15 us (both operands, launches, first and last steps), the
-    //           chunks, 8.5e-6 us per entry (sorting and expanding it);
+    //   here    14 us (both operands, launches, first and last steps), the
+    //           chunks, 4e-6 us per entry (until the expanding warps bound it,
+    //           from about 15%);
     //   sparse  8.5 us and t_entry per entry.
     // And the number from which it is the more exact one: a sum of the sparse
     // kernel runs over a row, or over the part of it in one unit, and its
-    // error grows with that length (1.0e-7 at 50, 1.4e-7 at 110, 1.6e-7 at
-    // 200, 5.5e-7 at 2000), here it is 1.2e-7 to 1.4e-7 (1.7e-7 at 2000).
-    const double t_tc = 15.0 + imin(whole, cut);
-    if (t_entry <= 9e-6) return;
+    // error grows with that length (1.0e-7 at 50, 1.4e-7 at 110, 1.7e-7 at
+    // 120 to 200, 7.8e-7 at 2000), here it is 0.7e-7 to 1.6e-7.
+    const double t_tc = 14.0 + imin(whole, cut);
+    if (t_entry <= 5e-6) return;
     const int64_t nnz_min = imax<int64_t>(imax<int64_t>((int64_t)rows * 160, (int64_t)sparse_units * 128),
-                                          (int64_t)(1.05 * (t_tc - 8.5) / (t_entry - 8.5e-6)));
+                                          (int64_t)(1.05 * (t_tc - 8.5) / (t_entry - 4e-6)));
     // Where the sparse kernel turns out to be the better one, the launch that
     // follows it in vain costs 1.5 us (and the host 4): not where only the
     // densest matrices would gain.
@@ -607,12 +618,10 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
         p += st_align(bytes);
         return at;
     };
-    plan->prep.parts = reinterpret_cast<uint32_t *>(take((size_t)4 * capacity));
+    plan->prep.sorted = reinterpret_cast<float *>(take((size_t)4 * capacity));
     plan->prep.place = reinterpret_cast<uint16_t *>(take((size_t)2 * capacity));
-    plan->prep.xp = reinterpret_cast<__half *>(take((size_t)4 * n * st_ld(k)));
+    plan->prep.xp = reinterpret_cast<__nv_bfloat16 *>(take((size_t)6 * n * st_ld(k)));
     plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)));
-    plan->prep.wscale = reinterpret_cast<float *>(take((size_t)4 * rows));
-    plan->prep.xscale = reinterpret_cast<float *>(take((size_t)4 * chunks * ceil_div(n, n_tile / 4)));
     plan->prep.num_marks = ceil_div(rows, kTcGroup) + chunks * ceil_div(n, n_tile / 4);
     plan->prep.marks = reinterpret_cast<uint8_t *>(take((size_t)plan->prep.num_marks));
     plan->prep.counters = 2 * plan->tiles;
@@ -623,7 +632,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.chunks = chunks;
     plan->prep.width = n_tile / 4;
     plan->prep.vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-    if (!make_map16(&plan->map_x, plan->prep.xp, false, (int64_t)2 * n, k, plan->prep.ld, n_tile / 2, kStChunk)) return;
+    if (!make_map16(&plan->map_x, plan->prep.xp, true, (int64_t)3 * n, k, plan->prep.ld, n_tile / 2, kStChunk)) return;
     static std::atomic<int> ready256[64], ready128[64];
     if (!(n_tile == 256 ? pair_kernel_ready(spmm_tc_kernel<256>, ready256, st_smem<256>(), kStThreads, kStSplitRegs)
                         : pair_kernel_ready(spmm_tc_kernel<128>, ready128, st_smem<128>(), kStThreads, kStSplitRegs)))
@@ -641,12 +650,10 @@ int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t
     a.rows = rows;
     a.k = plan.prep.k;
     a.n = n;
-    a.parts = plan.prep.parts;
+    a.sorted = plan.prep.sorted;
     a.place = plan.prep.place;
     a.start = plan.prep.start;
     a.x = x;
-    a.wscale = plan.prep.wscale;
-    a.xscale = plan.prep.xscale;
     a.y = y;
     a.partial = plan.partial;
     a.cnt = plan.prep.cnt;

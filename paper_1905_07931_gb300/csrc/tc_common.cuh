@@ -71,6 +71,8 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(const void *p) {
     return d;
 }
 
+constexpr uint32_t kSmemDescHi = (1024 >> 4) | (1u << 14) | (2u << 29);   // its high word
+
 // Instruction descriptor, kind::tf32: D = F32, A = B = TF32, both K-major.
 constexpr uint32_t kTcIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcBN >> 3) << 17) |
                               ((uint32_t)(kTcBM >> 4) << 24);

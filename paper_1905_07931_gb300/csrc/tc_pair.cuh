@@ -51,6 +51,26 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
+// Bounded wait for a phase of a barrier, or for another role's giving up. The
+// thread sleeps in the barrier unit for up to a microsecond per look instead
+// of taking issue slots from the warps that work.
+constexpr unsigned kPairWaitLooks = 1u << 18;
+__device__ __forceinline__ bool pair_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
+    const uint32_t addr = smem_u32(bar);
+    for (unsigned i = 0; i < kPairWaitLooks; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(addr), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
 // Arrives on the barrier at this offset in both CTAs once every MMA issued
 // before by this thread is done.
 __device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
@@ -60,12 +80,17 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
         "h"((uint16_t)3)
         : "memory");
 }
-__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+// The operands by the low words of their matrix descriptors (the address in
+// units of 16 bytes and the part that is the same for all K-major operands of
+// 128-byte rows; smem_desc_sw128): offsets are added there in 32 bits, and the
+// high word is a constant.
+__device__ __forceinline__ uint32_t smem_desc_lo(const void *p) { return (uint32_t)smem_desc_sw128(p); }
+__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint32_t adesc_lo, uint32_t bdesc_lo, uint32_t idesc,
                                              uint32_t accumulate) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(tmem_d),
+        "r"(adesc_lo), "r"(bdesc_lo), "r"(idesc), "r"(accumulate), "n"(kSmemDescHi)
         : "memory");
 }
 

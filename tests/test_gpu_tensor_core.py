@@ -193,3 +193,61 @@ def test_product_beside_another_kernel(C):
             assert torch.equal(_bits(got), _bits(want))
         side.synchronize()
     assert ws.status()[0] == 0
+
+
+def _uniform(seed, lo, hi, *shape):
+    return 10.0 ** (lo + (hi - lo) * torch.rand(*shape, device="cuda", generator=_gen(seed)))
+
+
+@pytest.mark.parametrize("m,k,n", [(4096, 4096, 256), (1025, 4000, 333), (1300, 5000, 99)])
+@pytest.mark.parametrize("what", ["samples", "rows", "tiny"])
+def test_product_of_any_range(C, m, k, n, what):
+    """An element of Y is as exact as its own terms allow, whatever the magnitudes around them: samples of very
+    different scale in one batch, rows whose entries span 15 decades and meet features of the inverse scale, values down
+    to float32's least. Each within float32's summation bound for its terms."""
+    ws = C.Workspace(m, k, n)
+    dense, x = _weights(m, k, 0.2, 1), torch.randn(k, n, device="cuda", generator=_gen(2))
+    dy = torch.randn(m, n, device="cuda", generator=_gen(3))
+    if what == "samples":
+        s = _uniform(4, -30, 0, 1, n)
+        x, dy = x * s, dy * s
+    elif what == "rows":
+        s = _uniform(5, -15, 0, k)
+        dense, x = dense * s, x / s[:, None] * 1e-8
+    else:
+        dense = dense * 2.0 ** -122    # down to 2^-149, 27 binades, with features of 2^25
+        x, dy = x * 2.0 ** 25, dy * 2.0 ** 25
+    w = _csr(C, dense, ws, transposed=True)
+    y, dx = torch.full((m, n), float("nan"), device="cuda"), torch.full((k, n), float("nan"), device="cuda")
+    C.launch_count(reset=True)
+    C.spmm_fwd(w, x, y, ws)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    C.spmm_bwd_t(w, dy, dx, ws)
+    d = dense.double()
+    for got, a, b in ((y, d, x), (dx, d.T, dy)):
+        terms = (a != 0).sum(1, keepdim=True).double()
+        lim = (terms + 64) * U * (a.abs() @ b.double().abs()) + 2.0 ** -149
+        assert bool(((got.double() - a @ b.double()).abs() <= lim).all())
+    assert ws.status()[0] == 0
+
+
+@pytest.mark.parametrize("m,n", [(4096, 256), (1300, 99)])
+def test_product_with_one_feature(C, m, n):
+    """Sums of one term: a feature of 1 returns W's entry, any other one rounding of the product and the parts that are
+    left out (at most 2^-24 of it each)."""
+    k = 4096
+    ws = C.Workspace(m, k, n)
+    dense = _weights(m, k, 0.3, 6)
+    w = _csr(C, dense, ws)
+    at = torch.randperm(k, generator=torch.Generator().manual_seed(1))[:n].cuda()
+    x = torch.zeros(k, n, device="cuda")
+    x[at, torch.arange(n, device="cuda")] = 1
+    y = torch.empty(m, n, device="cuda")
+    C.launch_count(reset=True)
+    C.spmm_fwd(w, x, y, ws)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    assert torch.equal(y, dense[:, at])
+    f = torch.randn(n, device="cuda", generator=_gen(7))
+    C.spmm_fwd(w, x * f, y, ws)
+    ref = dense[:, at].double() * f.double()
+    assert bool(((y.double() - ref).abs() <= 2 * U * ref.abs()).all())
