@@ -648,11 +648,10 @@ static int spmm_dispatch(const SpmmShape &sh, const SpmmArgs &args, const SpmmTc
     SpmmWideArgs wide;
     static_cast<SpmmArgs &>(wide) = args;
     wide.tc = tc;
-    const size_t prep_smem = tc.nnz_min > 0 ? (size_t)(tc.chunks + 1) * 17 * sizeof(int32_t) : 0;
     const unsigned fg = (unsigned)ceil_div<int64_t>(threads, 256);
 #define CSRT_SPMM_CASE(VW, NV, G, KERNEL, ARGS)                                             \
     if (sh.vw == VW && sh.nv == NV && sh.g == G) {                                          \
-        launch_pdl(KERNEL, dim3(grid), dim3(kSpThreads), G < 32 ? (size_t)kNarrowSmem : prep_smem, s, ARGS); \
+        launch_pdl(KERNEL, dim3(grid), dim3(kSpThreads), G < 32 ? (size_t)kNarrowSmem : 0, s, ARGS);        \
         if (fix) launch_pdl(spmm_fixup_kernel<G * VW * NV>, dim3(fg), dim3(256), 0, s, args); \
         return fix ? 2 : 1;                                                                 \
     }

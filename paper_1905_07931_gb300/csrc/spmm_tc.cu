@@ -15,11 +15,14 @@
 // sparse kernel has 1.7e-7 to 7.8e-7 (rows of 120 to 2000 entries); layers whose
 // rows hold fewer than 160 entries on average keep the sparse kernel.
 //
-// W never exists densely in memory: the first kernel (spmm_tc.cuh) sorts its
-// entries by groups of 16 rows and chunks of 64 columns, and eight warps
-// of each CTA put a chunk's entries into the cleared shared-memory operand of
-// the MMA (6 bytes per entry instead of 4 per element: written out as dense
-// planes, a layer at 5% took 52 us instead of 48, at 50% 83 instead of 96).
+// W exists in no other form than its CSR arrays: the first kernel (spmm_tc.cuh)
+// notes where each row's 64-column chunks begin (4 bytes per row and chunk),
+// and eight warps of each CTA put a chunk's entries into the cleared
+// shared-memory operand of the MMA. (Copies of the entries, sorted by 16 rows and
+// 64 columns, 6 bytes per entry of the capacity, took the workspace of a
+// 4096 x 9216 layer at 256 columns from 52 to 276 MB; they were faster only
+// where several column tiles each expand a very dense W, 4096 x 4096 x 1024 at
+// 50% 223 against 278 us, and slower else, x 256 at 20% 70 against 65.)
 //
 // Work: (256-row tile, kN columns of X) x 64-column chunks, cut into one
 // contiguous range per CTA pair. A pair whose range covers part of a tile's
@@ -27,8 +30,17 @@
 // add the parts up in pair order (st_share). Where there are enough tiles for
 // the GPU no tile is cut.
 //
+// Measured (GB300; the sparse kernel's time in brackets), rows x inner x n:
+// 4096 x 4096 x 256 at 20% 65 us (160), at 50% 104 (387), x 1024 at 5% 142
+// (169), at 50% 278 (1530); 4096 x 9216 x 256 at 5% 87 (98), at 20% 122 (365).
 // The MMAs take 1.7 us per chunk (six products; 24 of K = 16), with the
-// operands and the reading back 1.9.
+// operands and the reading back 1.9. From about 15% the expanding warps bound
+// it (4096 x 4096 x 1024 at 50%: 3.9 us per chunk; without the entries past each
+// row's sixteenth 182 us in all): some 700 instructions per warp and chunk, one
+// at a time. More of them in flight did not help: four rounds asked for ahead,
+// which took registers from the warps that add up, 268 us at 50% and 154
+// instead of 143 at 5%. The first kernel takes 40 us at 50%, the partial sums
+// of cut tiles 7 (20 MB written and read in L2).
 //
 // Operands that the tensor cores can't take (values of 2^28 and more, infinities,
 // NaN, rows out of order or with an entry twice) are marked by the first kernel
@@ -60,8 +72,6 @@ struct StArgs {
     const int32_t *row_ptr, *col;
     const float *val;
     int32_t rows, k, n;
-    const float *sorted;
-    const uint16_t *place;
     const int32_t *start;
     const float *x;
     float *y, *partial;
@@ -382,47 +392,71 @@ __global__ void __launch_bounds__(kStThreads, 1)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kStExpandRegs));
         // An expanding warp: one group of 16 rows. Per chunk it clears their
         // 128 bytes in the three planes and puts the entries' parts at their
-        // places, 256 entries at a time. The next entries are asked for as
-        // soon as these are in place: their latency (1000 clocks under load)
-        // passes while the MMAs of the stages ahead run. The bounds of 31
-        // chunks lie in the lanes of one register.
+        // places: eight lanes to a row, four rows at a time, eight entries of
+        // every row per round. Two rounds are asked for as soon as the chunk
+        // before is in place, and the bounds of the rows' runs one chunk
+        // earlier: their latency (1000 clocks under load) passes while the MMAs
+        // of the stage ahead run.
         const int e = warp - 4;
         const int groups = (a.rows + kTcGroup - 1) / kTcGroup;
+        const int sub = lane & 7, quad = lane >> 3;
         int tile = (int)(u_begin / a.chunks), ch = (int)(u_begin % a.chunks);
-        int32_t ends = 0;
-        int ch_ends = 0;   // lane l of `ends`: start[ch_ends + l]
-        auto load_ends = [&]() {
+        // the next unit's bounds: lane r the first entry of row r, lane 16 + r its end
+        int64_t asked = u_begin;
+        auto next_bounds = [&]() -> int32_t {
+            if (asked >= u_end) return 0;
             const int g = (tile / a.tiles_n) * 16 + (int)rank * 8 + e;
-            ch_ends = ch;
-            ends = g < groups ? __ldg(a.start + (int64_t)g * (a.chunks + 1) + imin(ch + lane, a.chunks)) : 0;
+            const int32_t got = g < groups ? __ldg(a.start + ((int64_t)g * (a.chunks + 1) + ch) * kTcGroup + lane) : 0;
+            ++asked;
+            if (++ch == a.chunks) {
+                ch = 0;
+                ++tile;
+            }
+            return got;
         };
-        float val[8];
-        uint32_t place[8];
-        auto fetch = [&](int32_t i, int32_t hi) {
+        int32_t col[2][4];
+        float val[2][4];
+        auto fetch = [&](int32_t bounds, int round) {
 #pragma unroll
-            for (int h = 0; h < 8; ++h) {
-                const bool on = i + h * 32 + lane < hi;
-                val[h] = on ? __ldg(a.sorted + i + h * 32 + lane) : 0.f;
-                place[h] = on ? __ldg(a.place + i + h * 32 + lane) : 0xffffu;
+            for (int s = 0; s < 4; ++s) {
+                const int r = (s >> 1) * 8 + (s & 1) + quad * 2;
+                const int32_t lo = __shfl_sync(0xffffffffu, bounds, r) + round * 8 + sub;
+                const int32_t hi = __shfl_sync(0xffffffffu, bounds, 16 + r);
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const int32_t i = lo + o * 8;
+                    col[o][s] = i < hi ? __ldg(a.col + i) : -1;
+                    val[o][s] = i < hi ? __ldg(a.val + i) : 0.f;
+                }
             }
         };
-        load_ends();
-        int32_t lo = __shfl_sync(0xffffffffu, ends, 0), hi = __shfl_sync(0xffffffffu, ends, 1);
-        fetch(lo, hi);
+        // (column j of row r lies at r * 128 + (2 j ^ (r & 7) * 16): 128-byte swizzle)
+        const uint32_t first = smem_u32(smem) + (uint32_t)(e * (kTcGroup * 128) + quad * 256);
+        auto put = [&](uint32_t at0) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                __nv_bfloat162 part[3];
+                split_bf16(make_float2(val[0][s], val[1][s]), part[0], part[1], part[2]);
+                const uint32_t turn = (uint32_t)((s & 1) * 16 + quad * 32);
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const uint32_t at = at0 + (s >> 1) * 1024 + (s & 1) * 128 + (((uint32_t)col[o][s] * 2 & 126) ^ turn);
+                    const uint32_t w1 = *reinterpret_cast<const uint32_t *>(&part[0]);
+                    const uint32_t w2 = *reinterpret_cast<const uint32_t *>(&part[1]);
+                    const uint32_t w3 = *reinterpret_cast<const uint32_t *>(&part[2]);
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ge.s32 p, %4, 0;\n @p st.shared.u16 [%0], %1;\n"
+                        " @p st.shared.u16 [%0 + %5], %2;\n @p st.shared.u16 [%0 + %6], %3;\n}\n" ::"r"(at),
+                        "h"((uint16_t)(o ? w1 >> 16 : w1)), "h"((uint16_t)(o ? w2 >> 16 : w2)),
+                        "h"((uint16_t)(o ? w3 >> 16 : w3)), "r"(col[o][s]), "n"(kStASlice), "n"(2 * kStASlice)
+                        : "memory");
+                }
+            }
+        };
+        int32_t bounds = next_bounds(), bounds_n = next_bounds();
+        fetch(bounds, 0);
         int it = 0;
         for (int64_t u = u_begin; u < u_end; ++u, ++it) {
-            int32_t lo_n = 0, hi_n = 0;   // the next chunk's entries
-            if (u + 1 < u_end) {
-                if (++ch == a.chunks) {
-                    ch = 0;
-                    ++tile;
-                    load_ends();
-                } else if (ch - ch_ends == 31) {
-                    load_ends();
-                }
-                lo_n = __shfl_sync(0xffffffffu, ends, ch - ch_ends);
-                hi_n = __shfl_sync(0xffffffffu, ends, ch - ch_ends + 1);
-            }
             const int s = it % kStages;
             uint8_t *base = smem + s * kStage + e * (kTcGroup * 128);
             if (!__all_sync(0xffffffffu, pair_wait(empty + s, ((it / kStages) & 1) ^ 1, &s_abort))) break;
@@ -433,29 +467,19 @@ __global__ void __launch_bounds__(kStThreads, 1)
                     *reinterpret_cast<uint4 *>(base + p * kStASlice + i * 512 + lane * 16) = make_uint4(0, 0, 0, 0);
             }
             __syncwarp();
-            while (true) {
-#pragma unroll
-                for (int h = 0; h < 8; h += 2) {
-                    __nv_bfloat162 part[3];
-                    split_bf16(make_float2(val[h], val[h + 1]), part[0], part[1], part[2]);
-#pragma unroll
-                    for (int p = 0; p < 3; ++p) {
-                        uint8_t *at = base + p * kStASlice;
-                        if (place[h] != 0xffffu) *reinterpret_cast<__nv_bfloat16 *>(at + place[h]) = part[p].x;
-                        if (place[h + 1] != 0xffffu) *reinterpret_cast<__nv_bfloat16 *>(at + place[h + 1]) = part[p].y;
-                    }
-                }
-                lo += 256;
-                if (lo >= hi) break;
-                fetch(lo, hi);
+            put(first + s * kStage);
+            const int run = __shfl_sync(0xffffffffu, bounds, 16 | lane) - bounds;   // (of lanes under 16)
+            const int longest = __reduce_max_sync(0xffffffffu, lane < 16 ? run : 0);
+            for (int round = 2; round * 8 < longest; round += 2) {
+                fetch(bounds, round);
+                put(first + s * kStage);
             }
-            // (loads in flight would hold up the fence: the next chunk's come after it)
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(map_to_rank(full + s, 0));
-            fetch(lo_n, hi_n);
-            lo = lo_n;
-            hi = hi_n;
+            bounds = bounds_n;
+            fetch(bounds, 0);
+            bounds_n = next_bounds();
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kStEpiRegs));
@@ -544,12 +568,12 @@ __global__ void __launch_bounds__(kStThreads, 1)
 static size_t st_align(size_t v) { return (v + 255) / 256 * 256; }
 static int32_t st_ld(int32_t k) { return (int32_t)ceil_div<int64_t>(k, 8) * 8; }
 static int st_max_pairs() { return imax(1, num_sms() / 2); }
-// Entries, planes, scales and partial sums of a rows x k matrix of at most
-// `capacity` entries and n columns.
-static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int64_t capacity, int n_tile) {
+// Row starts, planes, marks, counters and partial sums of a rows x k matrix and n
+// columns.
+static size_t st_bytes(int32_t rows, int32_t k, int32_t n, int n_tile) {
     const int64_t chunks = ceil_div(k, kStChunk);
-    return st_align((size_t)4 * capacity) + st_align((size_t)2 * capacity) + st_align((size_t)6 * n * st_ld(k)) +
-           st_align((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)) +
+    return st_align((size_t)6 * n * st_ld(k)) +
+           st_align((size_t)4 * kTcGroup * ceil_div(rows, kTcGroup) * (chunks + 1)) +
            st_align((size_t)ceil_div(rows, kTcGroup) + chunks * ceil_div(n, n_tile / 4)) +
            st_align((size_t)8 * ceil_div(rows, 256) * ceil_div(n, n_tile)) + (size_t)st_max_pairs() * 4 * 128 * n_tile * sizeof(float) + 512;
 }
@@ -563,8 +587,7 @@ size_t spmm_tc_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
     if (max_n < kStMinN) return 0;
     const bool fwd = st_shape_ok(rows, cols), bwd = st_shape_ok(cols, rows);
     if (!fwd && !bwd) return 0;
-    const int64_t all = (int64_t)rows * cols;
-    const size_t f = fwd ? st_bytes(rows, cols, max_n, all, 256) : 0, b = bwd ? st_bytes(cols, rows, max_n, all, 256) : 0;
+    const size_t f = fwd ? st_bytes(rows, cols, max_n, 256) : 0, b = bwd ? st_bytes(cols, rows, max_n, 256) : 0;
     return imax(f, b) <= (size_t)1 << 30 ? imax(f, b) : 0;   // beyond a gigabyte: the sparse kernel alone
 }
 
@@ -574,7 +597,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     if (!st_shape_ok(rows, k) || n < kStMinN || ws == nullptr || !device_is_sm10x()) return;
     const int n_tile = n <= 128 ? 128 : 256;
     capacity = imin<int64_t>(capacity, (int64_t)rows * k);
-    if (ws_bytes < kWsReservedBytes + st_bytes(rows, k, n, capacity, n_tile)) return;
+    if (ws_bytes < kWsReservedBytes + st_bytes(rows, k, n, n_tile)) return;
     const int chunks = ceil_div(k, kStChunk);
     plan->n_tile = n_tile;
     plan->tiles_n = ceil_div(n, n_tile);
@@ -618,10 +641,8 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
         p += st_align(bytes);
         return at;
     };
-    plan->prep.sorted = reinterpret_cast<float *>(take((size_t)4 * capacity));
-    plan->prep.place = reinterpret_cast<uint16_t *>(take((size_t)2 * capacity));
     plan->prep.xp = reinterpret_cast<__nv_bfloat16 *>(take((size_t)6 * n * st_ld(k)));
-    plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * ceil_div(rows, kTcGroup) * (chunks + 1)));
+    plan->prep.start = reinterpret_cast<int32_t *>(take((size_t)4 * kTcGroup * ceil_div(rows, kTcGroup) * (chunks + 1)));
     plan->prep.num_marks = ceil_div(rows, kTcGroup) + chunks * ceil_div(n, n_tile / 4);
     plan->prep.marks = reinterpret_cast<uint8_t *>(take((size_t)plan->prep.num_marks));
     plan->prep.counters = 2 * plan->tiles;
@@ -650,8 +671,6 @@ int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t
     a.rows = rows;
     a.k = plan.prep.k;
     a.n = n;
-    a.sorted = plan.prep.sorted;
-    a.place = plan.prep.place;
     a.start = plan.prep.start;
     a.x = x;
     a.y = y;

@@ -1,7 +1,6 @@
 // Interface between the sparse products (spmm.cu) and their tensor-core path
 // (spmm_tc.cu), and the work of that path's first kernel: X is written out as
-// three bf16 planes, W's entries are sorted into the blocks in which the GEMM
-// expands them.
+// three bf16 planes, and of W's rows is noted where each 64 columns begin.
 #pragma once
 
 #include <cuda.h>
@@ -12,8 +11,8 @@
 namespace csrt {
 
 constexpr int kTcChunk = 64;        // columns of W (features) per step of the GEMM
-constexpr int kTcGroup = 16;        // rows whose entries of a chunk lie together
-constexpr int kTcMaxChunks = 256;
+constexpr int kTcGroup = 16;        // rows that a warp of the GEMM expands
+constexpr int kTcMaxChunks = 256;   // (up to here the path was measured)
 constexpr int32_t kTcNoColumn = 0x7fffffff;   // past the end of a row
 
 // What the first kernel of an eligible product needs: if the matrix holds at
@@ -21,9 +20,7 @@ constexpr int32_t kTcNoColumn = 0x7fffffff;   // past the end of a row
 // that follows, else it computes the product and that kernel leaves at once.
 struct SpmmTcPrep {
     int64_t nnz_min;     // 0: no tensor-core kernel follows
-    float *sorted;       // [capacity] the entries in that order
-    uint16_t *place;     // and each one's byte offset in its group's 16 x 128 byte block of the GEMM's operand
-    int32_t *start;      // [groups][chunks + 1] first entry of each group's chunk
+    int32_t *start;      // [groups][chunks + 1][16] first entry of each row in each chunk
     __nv_bfloat16 *xp;   // [3][n][ld] the parts of X transposed
     int32_t k, ld, chunks;
     int32_t width;       // columns of X that a block of threads takes at a time
@@ -53,12 +50,6 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
 int spmm_tc_launch(const SpmmTcPlan &plan, const int32_t *row_ptr, const int32_t *col, const float *val, int32_t rows,
                    const float *x, int32_t n, float *y, const float *bias, int32_t relu, const float *mask, void *ws,
                    cudaStream_t s);
-
-// Byte offset of column j of row r in a block of 16 rows of 128 bytes with
-// the 128-byte swizzle.
-__device__ __forceinline__ uint32_t tc_place(int r, int j) {
-    return (uint32_t)(r * 128 + (((j >> 3) ^ (r & 7)) << 4) + (j & 7) * 2);
-}
 
 // X's planes of one chunk (64 features) and `width` columns (64 or 32) by a
 // block of 256 threads: a lane holds the features 2 lane and 2 lane + 1 of its
@@ -106,20 +97,16 @@ __device__ __forceinline__ void spmm_tc_prep_x(const SpmmTcPrep &a, const float 
     if (threadIdx.x == 0) a.marks[marks_w + chunk * ((n + a.width - 1) / a.width) + block] = bad;
 }
 
-// W's entries of one group of 16 rows by a block of 256 threads, two rows per
-// warp. The group's entries keep their range of the CSR arrays, sorted by
-// chunk and then by row. Columns ascend along a row, so its chunks are runs:
-// a first pass notes where each begins (the entry whose predecessor lies in
-// an earlier chunk); the rows' counts of each chunk, added up, give every run
-// its place, kept as the difference from its place in the CSR; the second pass
-// stores the entries there. tab: [chunks + 1][17] words (17: rows of one chunk in different banks).
-// Rows whose columns don't ascend have no such runs, and of two entries of one
-// column the operand could hold only one: their group is marked and left (the
-// sparse kernels, which add up whatever a row stores, take any order). So is
-// that of a value which can't be split.
+// W's rows of one group of 16 by a block of 256 threads, two rows per warp.
+// Columns ascend along a row, so its chunks are runs of entries, whose starts
+// are stored (the entry whose predecessor lies in an earlier chunk). Rows whose
+// columns don't ascend have no such runs, and of two entries of one column the
+// operand could hold only one: their group is marked (the sparse kernels, which
+// add up whatever a row stores, take any order). So is that of a value which
+// can't be split.
 __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_t *__restrict__ row_ptr,
                                                const int32_t *__restrict__ col, const float *__restrict__ val,
-                                               int32_t rows, int32_t group, int32_t (*tab)[17]) {
+                                               int32_t rows, int32_t group) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the warp's two rows side by side, 128 entries of each per step, the next
     // step's on their way while this one's are worked on
@@ -131,6 +118,7 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
         end[q] = r < rows ? __ldg(row_ptr + r + 1) : 0;
         len = max(len, end[q] - beg[q]);
     }
+    int32_t *start = a.start + (int64_t)group * (a.chunks + 1) * kTcGroup + warp * 2;
     int32_t c[2][4];
     float w[2][4];
     auto load = [&](int32_t i0) {
@@ -168,74 +156,12 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
                 // mostly none or one (columns before `prev`: none)
                 const int last = min(cc[q][h] >> 6, a.chunks);
                 for (int ch = max(prev >> 6, -1) + 1; ch <= last; ++ch)
-                    tab[ch][warp * 2 + q] = min(i0 + h * 32 + lane, end[q] - beg[q]);
+                    start[ch * kTcGroup + q] = min(beg[q] + i0 + h * 32 + lane, end[q]);
                 before[q] = __shfl_sync(0xffffffffu, cc[q][h], 31);
             }
     }
-    load(0);
-    __shared__ int32_t s_sum[9];
-    const int32_t base = __ldg(row_ptr + group * kTcGroup);
     unfit = __syncthreads_or(unfit);
     if (threadIdx.x == 0) a.marks[group] = unfit;
-    if (unfit) return;
-    // thread = chunk: its rows' counts, the chunks' first entries by a block scan
-    {
-        const int ch = threadIdx.x;
-        int32_t n = 0;
-        if (ch < a.chunks) {
-#pragma unroll
-            for (int r = 0; r < kTcGroup; ++r) n += tab[ch + 1][r] - tab[ch][r];
-        }
-        int32_t incl = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) s_sum[warp] = incl;
-        // (each thread reads its successor's row of tab: all before any writes)
-        int32_t cnt[kTcGroup];
-#pragma unroll
-        for (int r = 0; r < kTcGroup; ++r) cnt[r] = ch < a.chunks ? tab[ch + 1][r] - tab[ch][r] : 0;
-        __syncthreads();
-        int32_t at = base + incl - n;
-#pragma unroll
-        for (int o = 0; o < 8; ++o)
-            if (o < warp) at += s_sum[o];
-        int32_t *out = a.start + (int64_t)group * (a.chunks + 1);
-        if (ch < a.chunks) {
-            out[ch] = at;
-#pragma unroll
-            for (int r = 0; r < kTcGroup; ++r) {
-                tab[ch][r] = at - tab[ch][r];   // place of the row's entry i: tab + i
-                at += cnt[r];
-            }
-            if (ch == a.chunks - 1) out[a.chunks] = at;
-        }
-    }
-    __syncthreads();
-    for (int32_t i0 = 0; i0 < len; i0 += 128) {
-        int32_t cc[2][4];
-        float ww[2][4];
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                cc[q][h] = c[q][h];
-                ww[q][h] = w[q][h];
-            }
-        if (i0 + 128 < len) load(i0 + 128);
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                if (cc[q][h] == kTcNoColumn) continue;
-                const int32_t p = tab[cc[q][h] >> 6][warp * 2 + q] + i0 + h * 32 + lane;
-                a.sorted[p] = ww[q][h];
-                a.place[p] = (uint16_t)tc_place(warp * 2 + q, cc[q][h] & 63);
-            }
-    }
-    __syncthreads();   // tab is free again
 }
 
 // Both operands by a grid of 256-thread blocks: groups of W's rows (the longer
@@ -243,12 +169,11 @@ __device__ __forceinline__ void spmm_tc_prep_w(const SpmmTcPrep &a, const int32_
 __device__ __forceinline__ void spmm_tc_prep(const SpmmTcPrep &a, const int32_t *__restrict__ row_ptr,
                                              const int32_t *__restrict__ col, const float *__restrict__ val,
                                              int32_t rows, const float *__restrict__ x, int32_t n) {
-    extern __shared__ int32_t s_tab[][17];   // [chunks + 1], allocated only where this path may run
     const int nb = (n + a.width - 1) / a.width;
     const int ws = (rows + kTcGroup - 1) / kTcGroup, xs = a.chunks * nb;
     const int grid = (int)gridDim.x, b = (int)blockIdx.x;
     for (int i = b * blockDim.x + threadIdx.x; i < a.counters; i += grid * blockDim.x) a.cnt[i] = 0;
-    for (int i = b; i < ws; i += grid) spmm_tc_prep_w(a, row_ptr, col, val, rows, i, s_tab);
+    for (int i = b; i < ws; i += grid) spmm_tc_prep_w(a, row_ptr, col, val, rows, i);
     // X by the blocks that had fewer groups to do
     const int busy = ws % grid, idle = grid - busy;
     if (busy && idle >= grid / 4) {

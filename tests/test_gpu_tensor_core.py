@@ -251,3 +251,9 @@ def test_product_with_one_feature(C, m, n):
     C.spmm_fwd(w, x * f, y, ws)
     ref = dense[:, at].double() * f.double()
     assert bool(((y.double() - ref).abs() <= 2 * U * ref.abs()).all())
+
+
+@pytest.mark.parametrize("rows,cols,n,most", [(4096, 9216, 256, 64), (4096, 4096, 1024, 72), (8192, 16384, 1024, 192)])
+def test_workspace_follows_the_operands(C, rows, cols, n, most):
+    """The workspace (megabytes) holds parts of X and sums, not copies of W for a matrix that is full."""
+    assert C.Workspace(rows, cols, n).nbytes <= most * 1e6
