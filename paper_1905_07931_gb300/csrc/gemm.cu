@@ -11,11 +11,10 @@
 //    convolution layers: 20 x 25 outputs summed over 73,728 columns) split the
 //    reduction over blocks and add the partial tiles in a fixed order.
 //  * CSRT_PREC_TF32: tcgen05 tensor cores (gemm_tc.cu).
-#include "common.cuh"
+#include "gemm_tile.cuh"
 
 namespace csrt {
 
-constexpr int kGBM = 64, kGBN = 64, kGBK = 16;
 constexpr int64_t kGemmScratchFloats = (int64_t)1 << 24;   // 64 MB cap on split-reduction partials
 
 struct GemmSplit {
@@ -51,50 +50,11 @@ __global__ void __launch_bounds__(256) gemm_nt_f32_kernel(const float *__restric
                                                           int32_t m, int32_t k, int32_t n, int32_t chunk,
                                                           float *__restrict__ out) {
     pdl_enter();
-    __shared__ float as[kGBK][kGBM + 4];
-    __shared__ float bs[kGBK][kGBN + 4];
-    const int tid = threadIdx.x;
-    const int ty = tid / 16, tx = tid % 16;
-    const int64_t i0 = (int64_t)blockIdx.y * kGBM, j0 = (int64_t)blockIdx.x * kGBN;
+    __shared__ GemmTileSmem smem;
     const int split = blockIdx.z;
     const int nb = split * chunk, ne = min(n, nb + chunk);
-    float acc[4][4] = {};
-    for (int c0 = nb; c0 < ne; c0 += kGBK) {
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {
-            const int idx = tid + l * 256;
-            const int r = idx / kGBK, kk = idx % kGBK;
-            const int c = c0 + kk;
-            as[kk][r] = (i0 + r < m && c < ne) ? __ldg(dy + (i0 + r) * n + c) : 0.f;
-            bs[kk][r] = (j0 + r < k && c < ne) ? __ldg(x + (j0 + r) * n + c) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < kGBK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                a[t] = as[kk][ty * 4 + t];
-                b[t] = bs[kk][tx * 4 + t];
-            }
-#pragma unroll
-            for (int p = 0; p < 4; ++p)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
-        }
-        __syncthreads();
-    }
-    float *o = out + (int64_t)split * m * k;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const int64_t i = i0 + ty * 4 + p;
-        if (i >= m) continue;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int64_t j = j0 + tx * 4 + q;
-            if (j < k) o[i * k + j] = acc[p][q];
-        }
-    }
+    gemm_nt_tile(dy, x, m, k, n, nb, ne, (int64_t)blockIdx.y * kGBM, (int64_t)blockIdx.x * kGBN, (int)threadIdx.x, smem,
+                 out, split, [] { __syncthreads(); });
 }
 
 __global__ void split_reduce_kernel(const float *__restrict__ part, int64_t count, int32_t splits,

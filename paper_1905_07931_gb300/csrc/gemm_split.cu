@@ -17,8 +17,8 @@
 // bits is then below the fused multiply-add chain's for every n.
 //
 //  split_rows_kernel       dY and X to their planes (bf16, [3][rows][ld]) in the
-//                          workspace, a warp per row; rows that hold a value of
-//                          2^60 or more, an infinity or a NaN are marked.
+//                          workspace, a warp per row; blocks of eight rows that hold
+//                          a value of 2^60 or more, an infinity or a NaN are marked.
 //  gemm_split_kernel       CTA pairs (cta_group::2) walk 256 x 256 tiles of G:
 //                          per 64 columns six 16 KB slices per CTA (three planes
 //                          of its 128 rows of dY and 128 rows of X) by TMA, per
@@ -26,8 +26,12 @@
 //                          in tensor memory alternate between chunks; sixteen
 //                          warps per CTA read them back and keep the sums of
 //                          their 32 rows x 64 columns in registers.
-// Entries of marked rows are computed again by the epilogue with the plain
-// float32 chain, so infinities and NaN give what they give there.
+// With any block marked the second kernel computes all of G in tiles of float32
+// multiply-adds instead (gemm_tile.cuh: the CUDA-core kernel's, chain for
+// chain), so infinities and NaN give what they give there, for the CUDA-core
+// kernel's price (4096 x 4096 x 256 383 us). Doing only the marked rows'
+// entries so, a serial sum per thread, took 17 ms where one sample marked all
+// rows, 0.7 ms for one NaN.
 //
 // What bounds it: six bf16 products per multiply-add; 4096 x 4096 x 256 is
 // 51.5 GFLOP of MMA, 27 us at the measured bf16 rate, and 3.4 waves of tiles
@@ -39,6 +43,7 @@
 // 64-byte operand rows (stages of 32 columns) ran 11% slower than 128-byte
 // ones, eight reading warps with 128 sums each (spilling) 10%, arrivals with
 // .release.cluster 17-24%.
+#include "gemm_tile.cuh"
 #include "tc_pair.cuh"
 
 namespace csrt {
@@ -67,8 +72,9 @@ constexpr uint32_t kGsIdesc = idesc_f16(1, 256, 256);
 struct GsArgs {
     float *g;
     int32_t m, k, n;
-    const float *dy, *x;             // the float32 operands (marked rows)
-    const uint8_t *bad_dy, *bad_x;   // marked rows
+    const float *dy, *x;             // the float32 operands
+    const uint8_t *marks;            // [num_marks] blocks of eight rows
+    int32_t num_marks;
     int32_t tiles_k, num_tiles;
     WsHeader *hdr;
 };
@@ -78,13 +84,13 @@ struct GsArgs {
 __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict__ dy, const float *__restrict__ x,
                                                          int32_t m, int32_t k, int32_t n, int32_t ld,
                                                          __nv_bfloat16 *__restrict__ pdy,
-                                                         __nv_bfloat16 *__restrict__ px, uint8_t *__restrict__ bad_dy,
-                                                         uint8_t *__restrict__ bad_x, int vec) {
+                                                         __nv_bfloat16 *__restrict__ px, uint8_t *__restrict__ marks,
+                                                         int vec) {
     pdl_enter();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the GEMM's set-up may begin
     const int lane = threadIdx.x & 31;
     int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (r >= (int64_t)m + k) return;
+    const int cols = r < (int64_t)m + k ? n : 0;   // (the last block may have warps to spare)
     const bool is_x = r >= m;
     if (is_x) r -= m;
     const int64_t rows = is_x ? k : m;
@@ -92,7 +98,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
     __nv_bfloat16 *dst = (is_x ? px : pdy) + r * ld;
     const int64_t plane = rows * ld;
     bool bad = false;
-    for (int c = lane * 8; c < n; c += 256) {
+    for (int c = lane * 8; c < cols; c += 256) {
         float v[8];
         if (vec && c + 8 <= n) {
             const float4 a = ldg_f4(src + c), b = ldg_f4(src + c + 4);
@@ -119,8 +125,19 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
 #pragma unroll
         for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4 *>(dst + q * plane + c) = *reinterpret_cast<uint4 *>(p[q]);
     }
-    const bool any = __any_sync(0xffffffffu, bad);
-    if (lane == 0) (is_x ? bad_x : bad_dy)[r] = any ? 1 : 0;
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) marks[blockIdx.x] = bad;
+}
+
+// G by float32 multiply-adds, two 64 x 64 tiles at a time per CTA.
+static __device__ __noinline__ void gs_plain(const GsArgs &a, uint8_t *smem) {
+    const int group = threadIdx.x >> 8;
+    if (group >= 2) return;
+    GemmTileSmem &s = reinterpret_cast<GemmTileSmem *>(smem)[group];
+    const int64_t tiles_k = (a.k + kGBN - 1) / kGBN, tiles = (int64_t)((a.m + kGBM - 1) / kGBM) * tiles_k;
+    for (int64_t t = (int64_t)blockIdx.x * 2 + group; t < tiles; t += (int64_t)gridDim.x * 2)
+        gemm_nt_tile(a.dy, a.x, a.m, a.k, a.n, 0, a.n, t / tiles_k * kGBM, t % tiles_k * kGBN, threadIdx.x & 255, s, a.g, 0,
+                     [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + group) : "memory"); });
 }
 
 __global__ void __launch_bounds__(kGsThreads, 1)
@@ -171,8 +188,13 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     // nothing before this reads or writes global memory: the set-up overlaps
     // the end of the split kernel, whose planes are complete from here on
     pdl_enter();
+    bool marked = false;
+    for (int i = threadIdx.x; i < a.num_marks; i += kGsThreads) marked |= a.marks[i] != 0;
+    marked = __syncthreads_or(marked);   // the same for every CTA
 
-    if (warp < kGsProd) {
+    if (marked) {
+        gs_plain(a, smem);
+    } else if (warp < kGsProd) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGsProdRegs));
     if (warp == 0) {
         if (lane == 0) {
@@ -313,25 +335,6 @@ __global__ void __launch_bounds__(kGsThreads, 1)
                     }
                 }
             }
-            // entries of marked rows: the float32 chain
-            const bool bad_row = row < a.m && a.bad_dy[row];
-            bool bad_col = false;
-#pragma unroll
-            for (int e = 0; e < kGsEpiCols / 32; ++e) {
-                const int64_t col = col0 + e * 32 + lane;
-                bad_col |= col < a.k && a.bad_x[col];
-            }
-            if (__any_sync(0xffffffffu, bad_row || bad_col)) {
-                __syncwarp();
-                const int cols = (int)imin<int64_t>(kGsEpiCols, a.k - col0);
-                for (int e = 0; e < cols; ++e)
-                    if (row < a.m && (bad_row || a.bad_x[col0 + e])) {
-                        const float *p = a.dy + row * a.n, *w = a.x + (col0 + e) * a.n;
-                        float s = 0.f;
-                        for (int c = 0; c < a.n; ++c) s = fmaf(__ldg(p + c), __ldg(w + c), s);
-                        a.g[row * a.k + col0 + e] = s;
-                    }
-            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -352,8 +355,8 @@ static size_t gs_align(size_t v) { return (v + 255) / 256 * 256; }
 
 // Scratch of an m x k gradient over n columns: the planes and the marks.
 static size_t gs_bytes(int64_t m, int64_t k, int32_t n) {
-    return gs_align((size_t)(6 * m * gs_ld(n))) + gs_align((size_t)(6 * k * gs_ld(n))) + gs_align((size_t)m) +
-           gs_align((size_t)k) + 256;
+    return gs_align((size_t)(6 * m * gs_ld(n))) + gs_align((size_t)(6 * k * gs_ld(n))) +
+           gs_align((size_t)ceil_div<int64_t>(m + k, 8)) + 256;
 }
 
 size_t gemm_split_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
@@ -387,8 +390,8 @@ int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_
     p += gs_align((size_t)6 * m * ld);
     __nv_bfloat16 *px = reinterpret_cast<__nv_bfloat16 *>(p);
     p += gs_align((size_t)6 * k * ld);
-    uint8_t *bad_dy = reinterpret_cast<uint8_t *>(p);
-    uint8_t *bad_x = bad_dy + gs_align((size_t)m);
+    uint8_t *marks = reinterpret_cast<uint8_t *>(p);
+    const int32_t num_marks = (int32_t)ceil_div<int64_t>((int64_t)m + k, 8);
     CUtensorMap ma, mb;
     if (!make_map16(&ma, pdy, true, (int64_t)3 * m, n, ld, 128, kGsStageCols) ||
         !make_map16(&mb, px, true, (int64_t)3 * k, n, ld, 128, kGsStageCols))
@@ -402,14 +405,13 @@ int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_
     a.n = n;
     a.dy = dy;
     a.x = x;
-    a.bad_dy = bad_dy;
-    a.bad_x = bad_x;
+    a.marks = marks;
+    a.num_marks = num_marks;
     a.tiles_k = tiles_k;
     a.num_tiles = tiles;
     a.hdr = static_cast<WsHeader *>(ws);
     const int vec = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(dy) | reinterpret_cast<uintptr_t>(x)) & 15) == 0;
-    launch_pdl(split_rows_kernel, dim3((unsigned)ceil_div<int64_t>((int64_t)m + k, 8)), dim3(256), 0, s, dy, x, m, k, n,
-               ld, pdy, px, bad_dy, bad_x, vec);
+    launch_pdl(split_rows_kernel, dim3((unsigned)num_marks), dim3(256), 0, s, dy, x, m, k, n, ld, pdy, px, marks, vec);
     launch_pair(gemm_split_kernel, (unsigned)(2 * pairs), kGsThreads, kGsSmem, s, ma, mb, a);
     count_launch(2);
     *handled = true;

@@ -257,3 +257,40 @@ def test_product_with_one_feature(C, m, n):
 def test_workspace_follows_the_operands(C, rows, cols, n, most):
     """The workspace (megabytes) holds parts of X and sums, not copies of W for a matrix that is full."""
     assert C.Workspace(rows, cols, n).nbytes <= most * 1e6
+
+
+def test_gradient_with_a_bad_sample_costs_a_float32_product(C):
+    """One sample of infinities marks every row: right, and at the price of the CUDA-core gradient (8 times the tensor
+    cores', measured) and not that of a serial sum per entry (350 times)."""
+    m = k = 4096
+    n = 256
+    ws = C.Workspace(m, k, n)
+    dy, x = torch.randn(m, n, device="cuda", generator=_gen(1)), torch.randn(k, n, device="cuda", generator=_gen(2))
+    x = x.abs()
+    g = torch.empty(m, k, device="cuda")
+    plain = _us(lambda: C.weight_grad_dense(dy, x, g, ws, precision=0))
+    dy[5:, 3] = float("inf")
+    assert _us(lambda: C.weight_grad_dense(dy, x, g, ws, precision=0)) < 25 * plain
+    assert bool((g[5:] == float("inf")).all())
+    ref, mag = dy[:5].double() @ x.double().T, dy[:5].double().abs() @ x.double().T
+    assert bool(((g[:5].double() - ref).abs() <= n * U * mag).all())
+    assert ws.status()[0] == 0
+
+
+@pytest.mark.parametrize("m,k,n", [(300, 520, 250), (257, 1027, 200), (64, 4096, 1024)])
+def test_gradient_of_marked_operands_is_the_chain(C, m, k, n):
+    """With a value that the tensor cores can't take, every entry is the float32 chain of the CUDA-core kernel, bit for
+    bit (which runs without a workspace)."""
+    ws = C.Workspace(m, k, n)
+    dy, x = torch.randn(m, n, device="cuda", generator=_gen(m)), torch.randn(k, n, device="cuda", generator=_gen(k))
+    dy[m - 1, n - 1] = 2.0 ** 100
+    g, want = torch.full((m, k), float("nan"), device="cuda"), torch.full((m, k), float("nan"), device="cuda")
+    C.launch_count(reset=True)
+    C.weight_grad_dense(dy, x, g, ws, precision=0)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    ws.nbytes = 256     # no room for the parts
+    if n <= 512:        # (longer sums over few outputs need the workspace, and are added in slices)
+        C.weight_grad_dense(dy, x, want, ws, precision=0)
+        assert torch.equal(_bits(g), _bits(want))
+    ref, mag = dy.double() @ x.double().T, dy.double().abs() @ x.double().abs().T
+    assert bool(((g.double() - ref).abs() <= n * U * mag).all())
