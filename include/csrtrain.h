@@ -68,8 +68,10 @@ extern "C" {
 #define CSRT_DEV_INVALID 8    /* csrt_validate_csr found a broken invariant */
 
 /* weight_grad_dense precision. */
-#define CSRT_PREC_FP32 0      /* float32 accuracy: FMA on the CUDA cores, or float32 factors split into
-                                 three bf16 parts on tcgen05 (error below the FMA chain's) */
+#define CSRT_PREC_FP32 0      /* float32 accuracy: FMA on the CUDA cores, or float32 factors as three bf16
+                                 parts each (all 24 bits) on tcgen05: over 32 samples and more an error
+                                 below the FMA chain's; where one sample makes up a sum, one rounding
+                                 and at most 2^-24 of it */
 #define CSRT_PREC_TF32 1      /* tcgen05 tensor cores, kind::tf32, float32 accumulate */
 
 /*
@@ -258,7 +260,8 @@ int spmm_fwd_noalloc_status(int32_t *flags, int32_t clear, void *stream);
  * CSRT_PREC_TF32 (operands rounded to TF32, float32 accumulation).
  * CSRT_PREC_FP32 uses the workspace, where it is large enough, for the bf16
  * parts of dY and X; without one every shape runs on the CUDA cores (long
- * reductions over few outputs need it, as before). */
+ * reductions over few outputs need it, as before). Operands with infinities,
+ * NaN or values of 2^28 and more take the CUDA cores' chains, at their price. */
 int weight_grad_dense(const float *dy, const float *x, int32_t m, int32_t k, int32_t n,
                       float *g, int32_t precision, void *ws, size_t ws_bytes, void *stream);
 

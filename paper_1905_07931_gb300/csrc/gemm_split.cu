@@ -1,31 +1,27 @@
 // Dense weight gradient G = dY X^T in float32 accuracy on the tensor cores.
 //
-// Every float32 factor is the sum of three bf16 parts, x = x1 + x2 + x3 with
-// 8 significant bits each (round to nearest of what is left, so |x2| <= 2^-9
-// |x|, |x3| <= 2^-18 |x| and the sum is exact up to 2^-26 |x|). The product
-// is taken as x1 y1 + x1 y2 + x2 y1 + x2 y2 + x1 y3 + x3 y1; what is left out
-// is below 2^-26 |x y|, under float32's own rounding unit 2^-24.
-//
-// The accumulation must not lose what the split keeps. tcgen05.mma adds into
-// its float32 accumulator with truncation (measured: 2 bits beyond the
-// accumulator's last place are kept, the sum is cut toward zero), so a long
-// chain drifts: over 256 columns 2.3e-7 of the result against 1.1e-7 for a
-// chain of fused multiply-adds. Hence the reduction runs in chunks of 32
-// columns: in each the five small products come first (their truncations are
-// 2^-8 smaller), then the two steps of x1 y1, and the chunk's sum is added to
-// a float32 register accumulator with round to nearest. The error against 64
-// bits is then below the fused multiply-add chain's for every n.
+// Every float32 factor is the sum of three bf16 parts, all of its 24 bits at
+// every exponent below 2^28; six of the nine products of parts are taken, the
+// large one in sums of 64 columns that are added up with round to nearest
+// (split_bf16.cuh). The error against 64 bits is below that of a chain of fused
+// multiply-adds over the same columns (N(0, 1) over 256 columns 0.8e-7 against
+// 2.9e-7, positive factors 0.9e-7 against 2.5e-7, ReLU features and errors that
+// came through a ReLU 0.5e-7 against 1.4e-7), and where a single sample makes
+// up a sum, one rounding and the parts left out, 1.1e-7 at most against 6.0e-8.
+// (With one accumulator for all six products that was 1.6e-7, and parts that
+// are not scaled lost bits of values under 2^-110.)
 //
 //  split_rows_kernel       dY and X to their planes (bf16, [3][rows][ld]) in the
 //                          workspace, a warp per row; blocks of eight rows that hold
-//                          a value of 2^60 or more, an infinity or a NaN are marked.
+//                          a value of 2^28 or more, an infinity or a NaN are marked.
 //  gemm_split_kernel       CTA pairs (cta_group::2) walk 256 x 256 tiles of G:
 //                          per 64 columns six 16 KB slices per CTA (three planes
-//                          of its 128 rows of dY and 128 rows of X) by TMA, per
-//                          chunk 12 MMAs of M = 256, N = 256, K = 16; two accumulators
-//                          in tensor memory alternate between chunks; sixteen
-//                          warps per CTA read them back and keep the sums of
-//                          their 32 rows x 64 columns in registers.
+//                          of its 128 rows of dY and 128 rows of X) by TMA, 20
+//                          MMAs of M = 256, N = 256, K = 16 for the small products
+//                          and 4 for x1 y1, each kind with an accumulator of its
+//                          own in tensor memory; while the next columns' 20 run,
+//                          sixteen warps per CTA read x1 y1 back and add it to the
+//                          sums of their 32 rows x 64 columns in registers.
 // With any block marked the second kernel computes all of G in tiles of float32
 // multiply-adds instead (gemm_tile.cuh: the CUDA-core kernel's, chain for
 // chain), so infinities and NaN give what they give there, for the CUDA-core
@@ -35,21 +31,24 @@
 //
 // What bounds it: six bf16 products per multiply-add; 4096 x 4096 x 256 is
 // 51.5 GFLOP of MMA, 27 us at the measured bf16 rate, and 3.4 waves of tiles
-// run as 4. Measured (GB300, inputs in L2): 4096 x 4096 x 250 49 us (the
-// CUDA-core kernel 381), 4096 x 9216 x 256 91 us (830), 4096 x 4096 x 1024
-// 145 us (1464), 1000 x 4096 x 256 18 us (110). The MMAs alone take 0.91 us
-// per chunk and wave, with the operand loads and the reading back 1.0; a
-// wave's stores, which the next tile's first two chunks hide in part, 2-3 us.
-// 64-byte operand rows (stages of 32 columns) ran 11% slower than 128-byte
-// ones, eight reading warps with 128 sums each (spilling) 10%, arrivals with
+// run as 4. Measured (GB300, inputs in L2): 4096 x 4096 x 250 44 us (the
+// CUDA-core kernel 381), 4096 x 9216 x 256 79 us (831), 4096 x 4096 x 1024
+// 135 us (1466), 1000 x 4096 x 256 18 us (110), 4096 x 4096 x 32 23 us (55). The
+// MMAs alone take 1.8 us per 64 columns and wave, with the operand loads and the
+// reading back 1.9 to 2.0; a wave's stores, of which the next tile's first
+// columns hide part, 2-3 us; the look at the marks 1 us per call. x1 y1 read
+// after every 32 columns instead of 64: 53 us at 256 columns, 161 at 1024;
+// before the small products instead of after them: 2 to 4 us more; eight
+// reading warps with 128 sums each (spilling): 10%; arrivals with
 // .release.cluster 17-24%.
 #include "gemm_tile.cuh"
+#include "split_bf16.cuh"
 #include "tc_pair.cuh"
 
 namespace csrt {
 
-constexpr int kGsChunk = 32;                           // reduction columns per chunk sum
 constexpr int kGsStageCols = 64;                       // per pipeline stage: rows of 128 bytes
+static_assert(kGsStageCols == kSplitChunk, "a stage is a sum of x1 y1");
 constexpr int kGsSlice = 128 * kGsStageCols * 2;       // one plane of 128 rows: 16 KB
 constexpr int kGsStageBytes = 6 * kGsSlice;            // three planes of each operand
 constexpr int kGsStages = 2;
@@ -58,9 +57,10 @@ constexpr int kGsEpiCols = 64;
 constexpr int kGsProd = 4;                             // a warpgroup of producers (TMA, MMA, two idle)
 constexpr int kGsThreads = 32 * (kGsProd + kGsEpiWarps);
 // register split (ptxas gives the launch 640 x 96; it is found to hold the
-// shares before it is used): the sums (64), a block read back (32) and
-// addresses need more than 96 in the epilogue warps
-constexpr int kGsProdRegs = 32, kGsEpiRegs = 112;
+// shares before it is used): the sums (64), a block read back (16) and
+// addresses need more than 96 in the epilogue warps; with 32 instead of 64 the
+// producers spill
+constexpr int kGsProdRegs = 64, kGsEpiRegs = 104;
 constexpr int kGsSplitRegs = 128 * kGsProdRegs + 32 * kGsEpiWarps * kGsEpiRegs;
 static_assert(kGsSplitRegs <= kGsThreads * 96, "register split");
 constexpr int kGsTile = 256;
@@ -112,15 +112,8 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
             const float2 a = make_float2(v[e], v[e + 1]);
-            if (!(fabsf(a.x) < 0x1p60f) || !(fabsf(a.y) < 0x1p60f)) bad = true;
-            const __nv_bfloat162 b1 = __float22bfloat162_rn(a);
-            const float2 f1 = __bfloat1622float2(b1);
-            const float2 r1 = make_float2(a.x - f1.x, a.y - f1.y);
-            const __nv_bfloat162 b2 = __float22bfloat162_rn(r1);
-            const float2 f2 = __bfloat1622float2(b2);
-            p[0][e / 2] = b1;
-            p[1][e / 2] = b2;
-            p[2][e / 2] = __float22bfloat162_rn(make_float2(r1.x - f2.x, r1.y - f2.y));
+            if (!split_fits(a.x) || !split_fits(a.y)) bad = true;
+            split_bf16(a, p[0][e / 2], p[1][e / 2], p[2][e / 2]);
         }
 #pragma unroll
         for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4 *>(dst + q * plane + c) = *reinterpret_cast<uint4 *>(p[q]);
@@ -147,7 +140,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     float *epi = reinterpret_cast<float *>(smem + kGsStages * kGsStageBytes);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kGsStages * kGsStageBytes + kGsEpiWarps * kGsStageOut);
     uint64_t *empty = full + kGsStages;
-    uint64_t *accf = empty + kGsStages;   // [2] chunk sums ready
+    uint64_t *accf = empty + kGsStages;   // [2] the accumulator of x1 y1, that of the small products: ready
     uint64_t *acce = accf + 2;            // [2] read back (the leader's: all warps of both CTAs)
     uint64_t *fin = acce + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
@@ -157,7 +150,6 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     const uint32_t rank = cluster_rank();
     const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const int num_kb = (a.n + kGsStageCols - 1) / kGsStageCols;
-    const int num_ch = (a.n + kGsChunk - 1) / kGsChunk;
 
     if (threadIdx.x == 0) {
         s_abort = 0;
@@ -204,7 +196,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
                 const int k0 = (t % a.tiles_k) * kGsTile + (int)rank * 128;
                 for (int kb = 0; kb < num_kb; ++kb, ++it) {
                     const int s = it % kGsStages;
-                    if (!mbar_wait_or_abort(empty + s, ((it / kGsStages) & 1) ^ 1, &s_abort)) break;
+                    if (!pair_wait(empty + s, ((it / kGsStages) & 1) ^ 1, &s_abort)) break;
                     if (rank == 0) mbar_expect_tx(full + s, 2 * kGsStageBytes);
                     const uint32_t bar = map_to_rank(full + s, 0);
                     uint8_t *st = smem + s * kGsStageBytes;
@@ -222,31 +214,40 @@ __global__ void __launch_bounds__(kGsThreads, 1)
         }
     } else if (warp == 1) {
         if (rank == 0 && lane == 0) {
-            int it = 0, ch = 0;
+            int it = 0;
+            uint32_t turn = 0;   // bits 0 and 1: parity of the two accumulators
             for (int t = pair; t < a.num_tiles && !s_abort; t += pairs) {
                 for (int kb = 0; kb < num_kb; ++kb, ++it) {
-                    const int s = it % kGsStages;
-                    const uint8_t *st = smem + s * kGsStageBytes;
-                    if (!mbar_wait_or_abort(full + s, (it / kGsStages) & 1, &s_abort)) break;
+                    const int s = it % kGsStages, in_flush = kb % kSplitFlush;
+                    // steps of 16 columns (the last stage's columns past n are zero)
+                    const int steps = imin(kGsStageCols, a.n - kb * kGsStageCols + 15) / 16;
+                    if (!pair_wait(full + s, (it / kGsStages) & 1, &s_abort)) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int halves = imin(2, num_ch - 2 * kb);
-                    for (int hf = 0; hf < halves; ++hf, ++ch) {
-                        const int b = ch & 1;
-                        if (!mbar_wait_or_abort(acce + b, ((ch >> 1) & 1) ^ 1, &s_abort)) break;
+                    const uint32_t da = smem_desc_lo(smem + s * kGsStageBytes), db = da + (3 * kGsSlice >> 4);
+                    if (in_flush == 0) {
+                        if (!pair_wait(acce + 1, (turn >> 1) ^ 1, &s_abort)) break;
+                        turn ^= 2;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t d = tmem + (uint32_t)(b * 256);
-                        // planes of (dY, X): the small products first
-                        const int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
-#pragma unroll
-                        for (int q = 0; q < 6; ++q)
-#pragma unroll
-                            for (int k = 0; k < kGsChunk / 16; ++k)
-                                mma_f16_pair(d, smem_desc_lo(st + pa[q] * kGsSlice + hf * 64 + k * 32),
-                                             smem_desc_lo(st + (3 + pb[q]) * kGsSlice + hf * 64 + k * 32), kGsIdesc,
-                                             (q > 0 || k > 0) ? 1u : 0u);
-                        if (hf == halves - 1) mma_commit_pair(empty + s);
-                        mma_commit_pair(accf + b);
                     }
+                    // the small products first (while they run, the sum of x1 y1
+                    // before is read): parts of dY and of X by steps of four bits
+#pragma unroll 1
+                    for (int q = 0; q < 20; q += 4) {
+                        const uint32_t qa = da + (kSplitPartsA >> q & 3) * (kGsSlice >> 4);
+                        const uint32_t qb = db + (kSplitPartsB >> q & 3) * (kGsSlice >> 4);
+#pragma unroll
+                        for (int k = 0; k < kGsStageCols / 16; ++k)
+                            if (k < steps) mma_f16_pair(tmem + 256, qa + k * 2, qb + k * 2, kGsIdesc, k > 0 ? 1 : in_flush | q);
+                    }
+                    if (!pair_wait(acce, (turn & 1) ^ 1, &s_abort)) break;
+                    turn ^= 1;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                    for (int k = 0; k < kGsStageCols / 16; ++k)
+                        if (k < steps) mma_f16_pair(tmem, da + k * 2, db + k * 2, kGsIdesc, k > 0);
+                    mma_commit_pair(accf);
+                    mma_commit_pair(empty + s);
+                    if (in_flush == kSplitFlush - 1 || kb == num_kb - 1) mma_commit_pair(accf + 1);
                 }
             }
             asm volatile(
@@ -261,29 +262,36 @@ __global__ void __launch_bounds__(kGsThreads, 1)
         const int h = (warp - kGsProd) >> 2;     // column quarter of the tile
         const uint32_t acce0 = map_to_rank(acce, 0), acce1 = map_to_rank(acce + 1, 0);
         float *xb = epi + (warp - kGsProd) * (kGsStageOut / 4);
-        int it = 0;
+        int sums = 0, flushes = 0;
         for (int t = pair; t < a.num_tiles; t += pairs) {
             const int64_t row = (int64_t)(t / a.tiles_k) * kGsTile + rank * 128 + q * 32 + lane;
             const int64_t col0 = (int64_t)(t % a.tiles_k) * kGsTile + h * kGsEpiCols;
             float acc[kGsEpiCols];
+#pragma unroll
+            for (int c = 0; c < kGsEpiCols; ++c) acc[c] = 0.f;
             bool ok = true;
-            for (int kb = 0; kb < num_ch; ++kb, ++it) {
-                const int b = it & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait_or_abort(accf + b, (it >> 1) & 1, &s_abort));
-                if (!ok) break;
+            // (b = 0: the accumulator of x1 y1; 1: that of the small products)
+            auto add_up = [&](int b, int times) {
+                ok = __all_sync(0xffffffffu, pair_wait(accf + b, times & 1, &s_abort));
+                if (!ok) return;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int c = 0; c < kGsEpiCols; c += 32) {
-                    uint32_t r[32];
-                    tmem_ld_32cols(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256 + h * kGsEpiCols + c), r);
+                for (int c = 0; c < kGsEpiCols; c += 16) {
+                    uint32_t r[16];
+                    tmem_ld_16cols(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 256 + h * kGsEpiCols + c), r);
 #pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        acc[c + e] = kb == 0 ? __uint_as_float(r[e]) : acc[c + e] + __uint_as_float(r[e]);
+                    for (int e = 0; e < 16; ++e) acc[c + e] += __uint_as_float(r[e]);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(b ? acce1 : acce0);
+            };
+            for (int i = 1; i <= num_kb && ok; ++i) {
+                add_up(0, sums++);
+                if (ok && (i % kSplitFlush == 0 || i == num_kb)) add_up(1, flushes++);
             }
+#pragma unroll
+            for (int c = 0; c < kGsEpiCols; ++c) acc[c] *= kSplitDown;
             if (!ok) break;
             if (a.k % 8 == 0 && (reinterpret_cast<uintptr_t>(a.g) & 31) == 0) {
                 // lane = row holds 64 columns; groups of four lanes exchange
@@ -368,18 +376,19 @@ size_t gemm_split_scratch_bytes(int32_t rows, int32_t cols, int32_t max_n) {
 int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_t n, float *g, void *ws,
                    size_t ws_bytes, cudaStream_t s, bool *handled) {
     *handled = false;
-    // under 32 columns a chain of multiply-adds is as exact (16 columns: 4.3e-8
-    // against 4.7e-8) and its time is launch latency either way
-    if (m < 64 || k < 64 || n < kGsChunk || !device_is_sm10x()) return CSRT_OK;
+    // under 32 columns a chain of multiply-adds is as exact and its time is
+    // launch latency either way
+    if (m < 64 || k < 64 || n < 32 || !device_is_sm10x()) return CSRT_OK;
     if (ws == nullptr || ws_bytes < kWsReservedBytes + gs_bytes(m, k, n)) return CSRT_OK;
     const int tiles_k = (int)ceil_div<int64_t>(k, kGsTile);
     const int tiles = (int)ceil_div<int64_t>(m, kGsTile) * tiles_k;
     const int pairs = imin(tiles, imax(1, num_sms() / 2));
     // Where the CUDA-core kernel is still faster: small outputs, few columns.
     // Both times fitted to measurements on GB300 (microseconds; the split
-    // GEMM within 15% over 64..4096 x 64..9216 x 32..1024, the CUDA-core
-    // kernel, a latency per column or its 22 TFLOP/s, likewise).
-    const double waves = (double)ceil_div(tiles, pairs), chunks = (double)ceil_div(n, kGsChunk);
+    // GEMM's over 64..4096 x 64..9216 x 32..1024 is met or up to 19% above what
+    // it takes, the CUDA-core kernel's, a latency per column or its 22 TFLOP/s,
+    // within 15%).
+    const double waves = (double)ceil_div(tiles, pairs), chunks = (double)ceil_div(n, 32);
     const double t_split = 9.5 + waves * (2.5 + 1.0 * chunks);
     const double t_fma = imax(2.6 + 0.1 * imin(n, 512), 2.0 * m * k * n / 22e6);
     if (t_split > t_fma) return CSRT_OK;

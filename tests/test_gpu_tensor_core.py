@@ -294,3 +294,42 @@ def test_gradient_of_marked_operands_is_the_chain(C, m, k, n):
         assert torch.equal(_bits(g), _bits(want))
     ref, mag = dy.double() @ x.double().T, dy.double().abs() @ x.double().abs().T
     assert bool(((g.double() - ref).abs() <= n * U * mag).all())
+
+
+@pytest.mark.parametrize("m,k,n", [(300, 520, 250), (513, 1027, 600), (4096, 4096, 256)])
+@pytest.mark.parametrize("what", ["tiny", "samples", "large"])
+def test_gradient_of_any_range(C, m, k, n, what):
+    """Values down to float32's least against large ones, samples of very different scale, values up to 2^28: within
+    float32's summation bound for the terms of each entry."""
+    ws = C.Workspace(m, k, n)
+    dy, x = torch.randn(m, n, device="cuda", generator=_gen(1)), torch.randn(k, n, device="cuda", generator=_gen(2))
+    if what == "tiny":
+        dy, x = dy * 2.0 ** -122, x * 2.0 ** 25
+    elif what == "samples":
+        dy = dy * _uniform(3, -30, 0, 1, n)
+    else:
+        x = x * 2.0 ** 25
+    g = torch.full((m, k), float("nan"), device="cuda")
+    C.launch_count(reset=True)
+    C.weight_grad_dense(dy, x, g, ws, precision=0)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    ref, mag = dy.double() @ x.double().T, dy.double().abs() @ x.double().abs().T
+    # the truncated steps of 64 columns (8 U), the alignment of their products (8 U), the sums' roundings, the parts left out
+    lim = (n // 64 + 20) * U * mag + 2.0 ** -149
+    assert bool(((g.double() - ref).abs() <= lim).all())
+    assert ws.status()[0] == 0
+
+
+@pytest.mark.parametrize("m,k,n", [(300, 520, 250), (2000, 1030, 97)])
+def test_gradient_of_one_sample(C, m, k, n):
+    """A batch of which one sample counts (the others' errors are zero): one rounding of each product and the parts that
+    are left out, at most 2^-24 of it each."""
+    ws = C.Workspace(m, k, n)
+    dy, x = torch.zeros(m, n, device="cuda"), torch.randn(k, n, device="cuda", generator=_gen(2))
+    dy[:, n // 2] = torch.randn(m, device="cuda", generator=_gen(1))
+    g = torch.full((m, k), float("nan"), device="cuda")
+    C.launch_count(reset=True)
+    C.weight_grad_dense(dy, x, g, ws, precision=0)
+    assert C.launch_count() == 2, "a shape of the tensor-core path"
+    ref = dy.double() @ x.double().T
+    assert bool(((g.double() - ref).abs() <= 2 * U * ref.abs()).all())
