@@ -1216,7 +1216,7 @@ int weight_grad_sddmm(const csrt_csr *w, const float *dy, const float *x, int32_
     a.x = x;
     a.n = n;
     a.out = g_nnz;
-    static int cache[64][3][6][4];
+    static int cache[64][3][6][4][4];   // warps per SM, by device, vector, lanes, vectors per lane and form
     int dev = 0;
     CSRT_CHECK_CUDA(cudaGetDevice(&dev));
     CSRT_ARG(dev >= 0 && dev < 64, "device ordinal %d out of range", dev);
@@ -1224,6 +1224,7 @@ int weight_grad_sddmm(const csrt_csr *w, const float *dy, const float *x, int32_
     while ((1 << lg) < g) ++lg;
     while ((1 << lnv) < nv) ++lnv;
     void (*kern)(SddmmArgs) = nullptr;
+    int form = 0;   // of a wide kernel: one column tile, several, one filled, several filled
 #define CSRT_SDDMM_CASE(VW, G) \
     if (vw == VW && g == G) kern = sddmm_kernel<VW, 1, G>;
     CSRT_SDDMM_CASE(4, 1) CSRT_SDDMM_CASE(4, 2) CSRT_SDDMM_CASE(4, 4) CSRT_SDDMM_CASE(4, 8) CSRT_SDDMM_CASE(4, 16)
@@ -1235,12 +1236,19 @@ int weight_grad_sddmm(const csrt_csr *w, const float *dy, const float *x, int32_
     CSRT_SDDMM_CASE(4, 1) CSRT_SDDMM_CASE(4, 2) CSRT_SDDMM_CASE(2, 1) CSRT_SDDMM_CASE(2, 2) CSRT_SDDMM_CASE(2, 4)
     CSRT_SDDMM_CASE(1, 2) CSRT_SDDMM_CASE(1, 4) CSRT_SDDMM_CASE(1, 8)
 #undef CSRT_SDDMM_CASE
-    if (n > 256)
+    if (n > 256) {
+        form = 1;
         kern = vw == 4 ? sddmm_wide_kernel<4, 2, true> : vw == 2 ? sddmm_wide_kernel<2, 4, true> : sddmm_wide_kernel<1, 8, true>;
-    if (vw == 4 && n == 128) kern = sddmm_wide_kernel<4, 1, false, true>;
-    if (vw == 4 && n % 256 == 0) kern = n == 256 ? sddmm_wide_kernel<4, 2, false, true> : sddmm_wide_kernel<4, 2, true, true>;
-    // (the forms of a wide kernel have the same launch bounds)
-    int &wps = cache[dev][vw == 4 ? 2 : vw - 1][lg][lnv];
+    }
+    if (vw == 4 && n == 128) {
+        form = 2;
+        kern = sddmm_wide_kernel<4, 1, false, true>;
+    }
+    if (vw == 4 && n % 256 == 0) {
+        form = n == 256 ? 2 : 3;
+        kern = n == 256 ? sddmm_wide_kernel<4, 2, false, true> : sddmm_wide_kernel<4, 2, true, true>;
+    }
+    int &wps = cache[dev][vw == 4 ? 2 : vw - 1][lg][lnv][form];
     CSRT_ARG(kern != nullptr, "sddmm: no kernel for vw=%d nv=%d g=%d", vw, nv, g);
     // 2..16 lanes per entry: the per-warp ring of column indices in shared memory
     const size_t smem = (g > 1 && g < 32) ? (size_t)(kSpThreads / 32) * kSdStages * kSdChunk * sizeof(int32_t) : 0;

@@ -333,3 +333,22 @@ def test_gradient_of_one_sample(C, m, k, n):
     assert C.launch_count() == 2, "a shape of the tensor-core path"
     ref = dy.double() @ x.double().T
     assert bool(((g.double() - ref).abs() <= 2 * U * ref.abs()).all())
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 16, 33, 66, 127, 128, 129, 255, 256, 257, 300, 512, 1023, 1024])
+def test_sddmm_of_any_number_of_units(C, n):
+    """The gradient at the stored entries does not depend on how many units the entries are cut into: the same bits for
+    a capacity of the entries alone (a unit each) and of the dense matrix (all the GPU holds)."""
+    m, k = 37, 3000
+    dense = _weights(m, k, 0.005, n)
+    dense[[0, 5, 6, m - 1]] = 0
+    dense[9, :700] = 1
+    dy, x = torch.randn(m, n, device="cuda", generator=_gen(1)), torch.randn(k, n, device="cuda", generator=_gen(2))
+    ws, nnz = C.Workspace(m, k, n), int((dense != 0).sum())
+    got = []
+    for capacity in (nnz, m * k):
+        g = torch.full((nnz + 5,), 7.0, device="cuda")
+        C.weight_grad_sddmm(_csr(C, dense, ws, capacity=capacity), dy, x, g, ws)
+        assert bool((g[nnz:] == 7).all())
+        got.append(g[:nnz])
+    assert torch.equal(_bits(got[0]), _bits(got[1]))
