@@ -935,13 +935,12 @@ __global__ void __launch_bounds__(kSpThreads, VW * NV >= 8 ? 2 : 3) sddmm_wide_k
     }
 }
 
-template <int VW, int NV, int G>
+template <int VW, int G>
 __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
     pdl_enter();
     constexpr int E = 32 / G;
-    constexpr int U = VW * NV >= 4 ? 4 : 8;
+    constexpr int U = VW >= 4 ? 4 : 8;
     constexpr int B = U * E;
-    constexpr int TN = G * VW * NV, kStride = G * VW;
     constexpr int R = U < G ? U : G;
     const int lane = threadIdx.x & 31, grp = lane / G, gl = lane % G;
     const int64_t gw = ((int64_t)blockIdx.x * kSpThreads + threadIdx.x) >> 5;
@@ -950,7 +949,7 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
     const int64_t per = ceil_div<int64_t>(nnz, a.units);
     const int64_t k0 = min(gw * per, nnz), k1 = min(k0 + per, nnz);
     if (k0 >= k1) return;
-    const int n_tiles = (int)ceil_div<int64_t>(a.n, TN);
+    const bool on = gl * VW < a.n;   // the lane holds columns of the one tile
 
     int row = row_of_entry(a.row_ptr, a.rows, k0);
     int wb = row;
@@ -962,16 +961,12 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
         }
         return __shfl_sync(0xffffffffu, rpl, r - wb);
     };
-    float dyv[NV][VW];
-    auto load_dy = [&](int r, int tt) {
+    float dyv[VW];
+    auto load_dy = [&](int r) {
+        if (on) unpack<VW>(ldv<VW>(a.dy + (int64_t)r * a.n + gl * VW), dyv);
+        else {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int c = tt * TN + gl * VW + v * kStride;
-            if (c < a.n) unpack<VW>(ldv<VW>(a.dy + (int64_t)r * a.n + c), dyv[v]);
-            else {
-#pragma unroll
-                for (int e = 0; e < VW; ++e) dyv[v][e] = 0.f;
-            }
+            for (int e = 0; e < VW; ++e) dyv[e] = 0.f;
         }
     };
     int cn[U];
@@ -983,8 +978,8 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
     };
 
     int64_t e_row = row_end(row);
-    if (n_tiles == 1) load_dy(row, 0);
-    if constexpr (G > 1 && G < 32) {
+    load_dy(row);
+    if constexpr (G > 1) {
         // 2..16 lanes per entry (one tile covers n): the unit's column indices
         // stream through a per-warp cp.async ring of kSdStages chunks of
         // kSdChunk entries, two chunks ahead of the one being consumed
@@ -1013,7 +1008,7 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
                 while (e_row <= kb) {   // the row holding entry kb (empty rows are passed over)
                     ++row;
                     e_row = row_end(row);
-                    load_dy(row, 0);
+                    load_dy(row);
                 }
                 const int64_t kn = imin<int64_t>(imin<int64_t>(kb + B, e_row), ce);
                 const int rem = (int)(kn - kb - grp);
@@ -1027,25 +1022,17 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
                     c[st] = ok[st] ? ring[off + st * E] : 0;
                     p[st] = 0.f;
                 }
-                typename Vec<VW>::T xv[U][NV];
+                typename Vec<VW>::T xv[U];
 #pragma unroll
                 for (int st = 0; st < U; ++st)
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        const int col = gl * VW + v * kStride;
-                        if (ok[st] && col < a.n) xv[st][v] = ldv<VW>(a.x + (int64_t)c[st] * a.n + col);
-                    }
+                    if (ok[st] && on) xv[st] = ldv<VW>(a.x + (int64_t)c[st] * a.n + gl * VW);
 #pragma unroll
                 for (int st = 0; st < U; ++st)
+                    if (ok[st] && on) {
+                        float f[VW];
+                        unpack<VW>(xv[st], f);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        const int col = gl * VW + v * kStride;
-                        if (ok[st] && col < a.n) {
-                            float f[VW];
-                            unpack<VW>(xv[st][v], f);
-#pragma unroll
-                            for (int e = 0; e < VW; ++e) p[st] = fmaf(dyv[v][e], f[e], p[st]);
-                        }
+                        for (int e = 0; e < VW; ++e) p[st] = fmaf(dyv[e], f[e], p[st]);
                     }
                 group_reduce_multi<U, G>(p, gl);
                 if (gl % (G / R) == 0) {
@@ -1064,13 +1051,14 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
         cp_async_wait<0>();
         return;
     }
+    // one lane per entry: column indices one batch ahead, in registers
     int64_t kb = k0;
     fetch(kb);
     while (kb < k1) {
         while (e_row <= kb) {   // the row holding entry kb (empty rows are passed over)
             ++row;
             e_row = row_end(row);
-            if (n_tiles == 1) load_dy(row, 0);
+            load_dy(row);
         }
         int c[U];
 #pragma unroll
@@ -1080,50 +1068,22 @@ __global__ void __launch_bounds__(kSpThreads, 3) sddmm_kernel(SddmmArgs a) {
         const int64_t kn = imin<int64_t>(kb + B, e_cur);
         if (kn < k1) fetch(kn);
         const int rem = (int)imin<int64_t>(e_cur - kb - grp, B);
-        bool ok[U];
+        typename Vec<VW>::T xv[U];
 #pragma unroll
-        for (int s = 0; s < U; ++s) ok[s] = s * E < rem;
-        float p[U];
-#pragma unroll
-        for (int s = 0; s < U; ++s) p[s] = 0.f;
-        for (int tt = 0; tt < n_tiles; ++tt) {
-            if (n_tiles > 1) load_dy(row, tt);
-            typename Vec<VW>::T xv[U][NV];
-#pragma unroll
-            for (int s = 0; s < U; ++s)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const int col = tt * TN + gl * VW + v * kStride;
-                    if (ok[s] && col < a.n) xv[s][v] = ldv<VW>(a.x + (int64_t)c[s] * a.n + col);
-                }
-#pragma unroll
-            for (int s = 0; s < U; ++s)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const int col = tt * TN + gl * VW + v * kStride;
-                    if (ok[s] && col < a.n) {
-                        float f[VW];
-                        unpack<VW>(xv[s][v], f);
-#pragma unroll
-                        for (int e = 0; e < VW; ++e) p[s] = fmaf(dyv[v][e], f[e], p[s]);
-                    }
-                }
-        }
+        for (int s = 0; s < U; ++s)
+            if (s * E < rem && on) xv[s] = ldv<VW>(a.x + (int64_t)c[s] * a.n + gl * VW);
         float *op = a.out + kb + grp;
-        if constexpr (G == 1) {
 #pragma unroll
-            for (int s = 0; s < U; ++s)
-                if (ok[s]) op[s * E] = p[s];
-        } else {
-            group_reduce_multi<U, G>(p, gl);
-            if (gl % (G / R) == 0) {
-                const int r = gl / (G / R);
+        for (int s = 0; s < U; ++s) {
+            if (s * E >= rem) continue;
+            float p = 0.f;
+            if (on) {
+                float f[VW];
+                unpack<VW>(xv[s], f);
 #pragma unroll
-                for (int b = 0; b < U / R; ++b) {
-                    const int s = b * R + r;
-                    if (s * E < rem) op[s * E] = p[b * R];
-                }
+                for (int e = 0; e < VW; ++e) p = fmaf(dyv[e], f[e], p);
             }
+            op[s * E] = p;
         }
         kb = kn;
     }
@@ -1226,7 +1186,7 @@ int weight_grad_sddmm(const csrt_csr *w, const float *dy, const float *x, int32_
     void (*kern)(SddmmArgs) = nullptr;
     int form = 0;   // of a wide kernel: one column tile, several, one filled, several filled
 #define CSRT_SDDMM_CASE(VW, G) \
-    if (vw == VW && g == G) kern = sddmm_kernel<VW, 1, G>;
+    if (vw == VW && g == G) kern = sddmm_kernel<VW, G>;
     CSRT_SDDMM_CASE(4, 1) CSRT_SDDMM_CASE(4, 2) CSRT_SDDMM_CASE(4, 4) CSRT_SDDMM_CASE(4, 8) CSRT_SDDMM_CASE(4, 16)
     CSRT_SDDMM_CASE(2, 1) CSRT_SDDMM_CASE(2, 2) CSRT_SDDMM_CASE(2, 4) CSRT_SDDMM_CASE(2, 8) CSRT_SDDMM_CASE(2, 16)
     CSRT_SDDMM_CASE(1, 1) CSRT_SDDMM_CASE(1, 2) CSRT_SDDMM_CASE(1, 4) CSRT_SDDMM_CASE(1, 8) CSRT_SDDMM_CASE(1, 16)
