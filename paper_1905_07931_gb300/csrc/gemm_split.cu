@@ -67,7 +67,7 @@ constexpr int kGsTile = 256;
 constexpr int kGsStageOut = 32 * 16 * 4;               // a 32 x 16 block on its way out
 constexpr int kGsSmem = kGsStages * kGsStageBytes + kGsEpiWarps * kGsStageOut + 1024 + 256;
 static_assert(kGsSmem <= 232448, "shared memory per block");
-constexpr uint32_t kGsIdesc = idesc_f16(1, 256, 256);
+constexpr uint32_t kGsIdesc = idesc_bf16(256, 256);
 
 struct GsArgs {
     float *g;
@@ -237,14 +237,14 @@ __global__ void __launch_bounds__(kGsThreads, 1)
                         const uint32_t qb = db + (kSplitPartsB >> q & 3) * (kGsSlice >> 4);
 #pragma unroll
                         for (int k = 0; k < kGsStageCols / 16; ++k)
-                            if (k < steps) mma_f16_pair(tmem + 256, qa + k * 2, qb + k * 2, kGsIdesc, k > 0 ? 1 : in_flush | q);
+                            if (k < steps) mma_bf16_pair(tmem + 256, qa + k * 2, qb + k * 2, kGsIdesc, k > 0 ? 1 : in_flush | q);
                     }
                     if (!pair_wait(acce, (turn & 1) ^ 1, &s_abort)) break;
                     turn ^= 1;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                     for (int k = 0; k < kGsStageCols / 16; ++k)
-                        if (k < steps) mma_f16_pair(tmem, da + k * 2, db + k * 2, kGsIdesc, k > 0);
+                        if (k < steps) mma_bf16_pair(tmem, da + k * 2, db + k * 2, kGsIdesc, k > 0);
                     mma_commit_pair(accf);
                     mma_commit_pair(empty + s);
                     if (in_flush == kSplitFlush - 1 || kb == num_kb - 1) mma_commit_pair(accf + 1);
@@ -402,8 +402,8 @@ int gemm_split_f32(const float *dy, const float *x, int32_t m, int32_t k, int32_
     uint8_t *marks = reinterpret_cast<uint8_t *>(p);
     const int32_t num_marks = (int32_t)ceil_div<int64_t>((int64_t)m + k, 8);
     CUtensorMap ma, mb;
-    if (!make_map16(&ma, pdy, true, (int64_t)3 * m, n, ld, 128, kGsStageCols) ||
-        !make_map16(&mb, px, true, (int64_t)3 * k, n, ld, 128, kGsStageCols))
+    if (!make_map_bf16(&ma, pdy, (int64_t)3 * m, n, ld, 128) ||
+        !make_map_bf16(&mb, px, (int64_t)3 * k, n, ld, 128))
         return CSRT_OK;
     static std::atomic<int> ready[64];
     if (!pair_kernel_ready(gemm_split_kernel, ready, kGsSmem, kGsThreads, kGsSplitRegs)) return CSRT_OK;

@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kStThreads, 1)
     }
     constexpr int kStages = st_stages<kN>(), kStage = st_stage<kN>(), kBSlice = st_bslice<kN>();
     constexpr int kCols = kN / 4;   // columns of an epilogue warp
-    constexpr uint32_t kIdesc = idesc_f16(1, 256, kN);
+    constexpr uint32_t kIdesc = idesc_bf16(256, kN);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStage);
@@ -365,14 +365,14 @@ __global__ void __launch_bounds__(kStThreads, 1)
                     const uint32_t qb = da + (3 * kStASlice >> 4) + (kSplitPartsB >> q & 3) * (kBSlice >> 4);
 #pragma unroll
                     for (int k = 0; k < kStChunk / 16; ++k)
-                        mma_f16_pair(tmem + kN, qa + k * 2, qb + k * 2, kIdesc, k > 0 ? 1 : in_flush | q);
+                        mma_bf16_pair(tmem + kN, qa + k * 2, qb + k * 2, kIdesc, k > 0 ? 1 : in_flush | q);
                 }
                 if (!pair_wait(acce, (turn >> 1 & 1) ^ 1, &s_abort)) break;
                 turn ^= 2;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                 for (int k = 0; k < kStChunk / 16; ++k)
-                    mma_f16_pair(tmem, da + k * 2, da + (3 * kStASlice >> 4) + k * 2, kIdesc, k > 0);
+                    mma_bf16_pair(tmem, da + k * 2, da + (3 * kStASlice >> 4) + k * 2, kIdesc, k > 0);
                 mma_commit_pair(accf);
                 ++in_flush;
                 mma_commit_pair(empty + st);
@@ -653,7 +653,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->prep.chunks = chunks;
     plan->prep.width = n_tile / 4;
     plan->prep.vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-    if (!make_map16(&plan->map_x, plan->prep.xp, true, (int64_t)3 * n, k, plan->prep.ld, n_tile / 2, kStChunk)) return;
+    if (!make_map_bf16(&plan->map_x, plan->prep.xp, (int64_t)3 * n, k, plan->prep.ld, n_tile / 2)) return;
     static std::atomic<int> ready256[64], ready128[64];
     if (!(n_tile == 256 ? pair_kernel_ready(spmm_tc_kernel<256>, ready256, st_smem<256>(), kStThreads, kStSplitRegs)
                         : pair_kernel_ready(spmm_tc_kernel<128>, ready128, st_smem<128>(), kStThreads, kStSplitRegs)))

@@ -1,5 +1,5 @@
 // Helpers of the tensor-core kernels that run on CTA pairs (tcgen05
-// cta_group::2, a cluster of two CTAs on one 256-row tile) with 16-bit
+// cta_group::2, a cluster of two CTAs on one 256-row tile) with bf16
 // operand planes: barriers of the pair, TMA loads that signal the leader's
 // barrier, matrix and instruction descriptors, 256-bit stores.
 //
@@ -14,7 +14,6 @@
 #include <atomic>
 
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include "tc_common.cuh"
 
@@ -85,7 +84,7 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
 // 128-byte rows; smem_desc_sw128): offsets are added there in 32 bits, and the
 // high word is a constant.
 __device__ __forceinline__ uint32_t smem_desc_lo(const void *p) { return (uint32_t)smem_desc_sw128(p); }
-__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint32_t adesc_lo, uint32_t bdesc_lo, uint32_t idesc,
+__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint32_t adesc_lo, uint32_t bdesc_lo, uint32_t idesc,
                                              uint32_t accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
@@ -94,11 +93,10 @@ __device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint32_t adesc_lo,
         : "memory");
 }
 
-// Instruction descriptor, kind::f16 with float32 accumulators, both operands
-// K-major: type 0 = f16, 1 = bf16.
-__host__ __device__ constexpr uint32_t idesc_f16(int type, int m, int n) {
-    return (1u << 4) | ((uint32_t)type << 7) | ((uint32_t)type << 10) | ((uint32_t)(n >> 3) << 17) |
-           ((uint32_t)(m >> 4) << 24);
+// Instruction descriptor, kind::f16: bf16 operands, both K-major, float32
+// accumulators.
+__host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 // Sixteen columns of this warp's 32 tensor-memory lanes.
@@ -126,21 +124,18 @@ __device__ __forceinline__ void ld_global_f8(const float *p, float (&v)[8]) {
                  : "memory");
 }
 
-// Row-major rows x cols matrix of 16-bit elements with row stride ld elements
-// (a multiple of 8): boxes of box_rows x 32 elements (64-byte swizzle) or x 64
-// (128-byte swizzle).
-inline bool make_map16(CUtensorMap *map, const void *base, bool bf16, int64_t rows, int64_t cols, int64_t ld,
-                       int box_rows, int box_cols) {
+// Row-major rows x cols matrix of bf16 with row stride ld elements (a multiple
+// of 8): boxes of box_rows x 64 elements, 128-byte swizzle.
+inline bool make_map_bf16(CUtensorMap *map, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
-                    const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 
