@@ -608,7 +608,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     // (microseconds; the partial sums take 4 us and 2.2 us for each eighth of
     // a tile's columns that a pair has to add up).
     const int max_pairs = st_max_pairs();
-    const double t_unit = n_tile == 256 ? 1.95 : 1.75;
+    const double t_unit = n_tile == 256 ? 1.85 : 1.75;
     const int cut_pairs = (int)imin<int64_t>(units, max_pairs);
     const double whole = (double)ceil_div(plan->tiles, max_pairs) * chunks * t_unit;
     const double cut = (double)ceil_div<int64_t>(units, cut_pairs) * t_unit + 4.0 +
@@ -616,12 +616,15 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     plan->whole = whole <= cut;
     plan->pairs = plan->whole ? ceil_div(plan->tiles, ceil_div(plan->tiles, max_pairs)) : cut_pairs;
     // The number of entries from which this path is the faster one: both
-    // times are fits to measurements over 512..9216 rows and columns, 1% to
-    // 50% and 100 to 1024 columns of X (within 15%):
+    // times are fits to measurements over 512..9216 rows and columns, 3% to
+    // 20% and 99 to 1024 columns of X (within 8%):
     //   here    14 us (both operands, launches, first and last steps), the
     //           chunks, 4e-6 us per entry (until the expanding warps bound it,
     //           from about 15%);
     //   sparse  8.5 us and t_entry per entry.
+    // Where the two meet, 0.95 of what they give is what was measured: 4096 x
+    // 4096 x 256 5.5%, x 1024 4.1%, 4096 x 9216 x 256 4.4% (at 5% 87 us against
+    // 98), 1300 x 5000 x 99 5.6%.
     // And the number from which it is the more exact one: a sum of the sparse
     // kernel runs over a row, or over the part of it in one unit, and its
     // error grows with that length (1.0e-7 at 50, 1.4e-7 at 110, 1.7e-7 at
@@ -629,7 +632,7 @@ void spmm_tc_plan(int32_t rows, int32_t k, int32_t n, int64_t capacity, const fl
     const double t_tc = 14.0 + imin(whole, cut);
     if (t_entry <= 5e-6) return;
     const int64_t nnz_min = imax<int64_t>(imax<int64_t>((int64_t)rows * 160, (int64_t)sparse_units * 128),
-                                          (int64_t)(1.05 * (t_tc - 8.5) / (t_entry - 4e-6)));
+                                          (int64_t)(0.95 * (t_tc - 8.5) / (t_entry - 4e-6)));
     // Where the sparse kernel turns out to be the better one, the launch that
     // follows it in vain costs 1.5 us (and the host 4): not where only the
     // densest matrices would gain.
