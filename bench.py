@@ -450,7 +450,7 @@ def record_traffic(csv_path: str, out_path: str) -> dict:
     if len(sp) >= 10:
         labels = ["spmm_fwd_bias_act[layer 0]", "spmm_fwd_bias_act[layer 1]", "spmm_fwd_bias_act[layer 2]",
                   "spmm_bwd_t_relu[layer 2]", "spmm_bwd_t_relu[layer 1]"]
-        srcs = ["spmm.cu", "spmm_tc.cu", "spmm_tc.cuh", "tc_pair.cuh", "common.cuh"]
+        srcs = ["spmm.cu", "spmm_tc.cu", "spmm_tc.cuh", "split_bf16.cuh", "tc_pair.cuh", "common.cuh"]
         for lab, call in zip(labels, sp[5:10]):
             rd = sum(k.get("dram__bytes_read.sum", 0.0) for k in call)
             wr = sum(k.get("dram__bytes_write.sum", 0.0) for k in call)

@@ -72,8 +72,10 @@ inline cudaStream_t as_stream(void *s) { return static_cast<cudaStream_t>(s); }
 // starts with pdl_enter(): griddepcontrol.wait returns once the previous
 // kernel has completed and its writes are visible. Launched without the
 // attribute, the instruction does nothing. (An explicit early
-// launch_dependents, which would let the next kernel's blocks wait on the
-// SMs during this kernel's last wave, measured slower on the training step.)
+// launch_dependents, which lets the next kernel's blocks wait on the SMs
+// during this kernel's last wave, measured slower on the training step; it
+// pays in front of the two tensor-core kernels of one block per SM, whose
+// set-up it hides: gemm_split.cu, spmm.cu.)
 __device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... P, typename... A>
